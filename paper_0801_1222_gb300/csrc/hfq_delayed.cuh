@@ -44,8 +44,9 @@ struct DelLayout {
   uint32_t off_stage, off_G, off_U, off_W, off_diag, off_gtile;
   size_t bytes;
   uint32_t off_gjb;  // the recompute's panel scratch (workspace in HBM), overlaying all but G
-  uint32_t off_rf;   // the Newton refinement's staging (1024-aligned; overlays the whole body,
-                     // a resident G included: G is kept in HBM while it runs)
+  uint32_t off_rf;   // the Newton refinement's staging (1024-aligned): after a resident G when
+                     // it fits there, else over the whole body
+  bool rf_keeps_G;   // it lies after the resident G (else G goes to HBM while it runs)
 };
 
 // product buffers of the TMA reduce flush: two halves of a tile, 64 rows x
@@ -84,11 +85,16 @@ __host__ __device__ inline size_t del_stage_bytes(int K, int L, int ub) {
   return (size_t)(2 + 2 * del_ublocks(L, ub)) * kTileN * KS * 2;
 }
 
+// Shared memory of the Newton refinement (hfq_refine.cuh): A's slice table
+// and a factor per row, or the update product's two stage buffers and three
+// factors per row, or the
+// particle-hole mirror's tiles (32 x 33 floats per warp), whichever is larger
 __host__ __device__ inline size_t rf_smem_need(int L) {
-  // the Newton refinement (hfq_refine.cuh): the larger of its two stage buffers of the residual product (A and H'
-  // slices) and GEMM2's (H' and E^T hi / lo parts)
-  const size_t g2 = (size_t)2 * 128 * kRf2KC * 2 + (size_t)2 * ((L + 15) / 16 * 16) * kRf2KC * 2;
-  return g2 > (size_t)kRfSmem ? g2 : (size_t)kRfSmem;
+  const size_t g1 = rf_tab_bytes(L) + (size_t)rf_nj(L) * 8 * 4;
+  const size_t g2 = 2 * (size_t)rf_stage2_bytes(L) + (size_t)rf_pad(L, 16) * 16;
+  const size_t mt = (size_t)(kDelNT / 32) * 32 * 33 * 4;
+  const size_t m = kRfHead + (g1 > g2 ? g1 : g2);
+  return m > mt ? m : mt;
 }
 
 // ns: spins the sweep keeps (2, or 1 for the G_up-only sweep): the panels and
@@ -145,6 +151,8 @@ __host__ __device__ inline DelLayout del_layout(int L, int K, bool resident, boo
   d.off_gjb = resident ? del_align(d.off_U, 128) : del_align(d.off_body + scratch, 128);
   if (!gj_smem && d.off_gjb + gj_blocked_bytes(L) > o) o = d.off_gjb + gj_blocked_bytes(L);
   d.off_rf = d.off_body;
+  d.rf_keeps_G = resident && refine && del_align(d.off_U, 1024) + rf_smem_need(L) <= kSmemCap;
+  if (d.rf_keeps_G) d.off_rf = del_align(d.off_U, 1024);
   if (refine && d.off_rf + rf_smem_need(L) > o) o = d.off_rf + rf_smem_need(L);
   d.bytes = o;
   return d;
@@ -225,9 +233,14 @@ struct TcState {
   uint32_t mbar;       // shared address of the MMA completion mbarrier
   uint32_t phase;      // parity of the next MMA completion
   int failed;          // a wait gave up: the tensor path is not used again
-  uint32_t cbar;       // shared address of the refinement's mbarriers: bulk copy into
-                       // stage buffer 0, 1, then MMA completion of buffer 0, 1 (8 bytes apart)
-  uint32_t cphase;     // their parities (bit b of the barrier at cbar + 8 b)
+  uint32_t cbar;       // shared address of the refinement's mbarriers (8 bytes apart): table copy,
+                       // the four H' buffers full, the four consumed, the two update stages consumed
+};
+
+// The refinement's counters, kept in shared memory between recomputes: H'
+// buffers and update stages used so far, table copies so far
+struct RfSync {
+  uint32_t cc, c2, ct;
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -309,18 +322,16 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t mbar, uint32_t phase) {
   return ok != 0;
 }
 
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Waits for the mbarrier phase with a one-second limit; false on timeout.
+// Waits for the mbarrier phase with a limit of 2^31 SM cycles (about a
+// second); false on timeout.  The limit is read from the SM's own clock, and
+// only once the phase was found incomplete: a read of the global timer costs
+// more than most of these waits.
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t mbar, uint32_t phase) {
-  const unsigned long long t0 = global_ns();
+  if (mbar_try_wait(mbar, phase)) return true;
+  const long long t0 = clock64();
   for (;;) {
     if (mbar_try_wait(mbar, phase)) return true;
-    if (global_ns() - t0 > 1000000000ull) return false;
+    if (clock64() - t0 > (1ll << 31)) return false;
   }
 }
 
@@ -349,7 +360,9 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
 }
 
 // Allocates kTmemCols TMEM columns (warp 0) and initialises the MMA
-// completion mbarrier s_mbar[0] and the refinement's four, s_mbar[1..4].
+// completion mbarrier s_mbar[0] and the refinement's eleven, s_mbar[1..11]
+// (the four "full" ones, 2 to 5, take one arrival per lane quarter and block of
+// eight contraction rows).
 __device__ inline void tc_setup(TcState* tc, uint32_t* s_tmem, unsigned long long* s_mbar,
                                 int* status) {
   (void)status;
@@ -361,8 +374,9 @@ __device__ inline void tc_setup(TcState* tc, uint32_t* s_tmem, unsigned long lon
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (threadIdx.x == 0) {
-    for (int b = 0; b < 5; ++b)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(s_mbar + b)) : "memory");
+    for (int b = 0; b < 12; ++b)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(s_mbar + b)), "r"(b >= 2 && b <= 5 ? 8 : 1)
+                   : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   tc_fence_before();
@@ -373,7 +387,6 @@ __device__ inline void tc_setup(TcState* tc, uint32_t* s_tmem, unsigned long lon
   tc->phase = 0;
   tc->failed = 0;
   tc->cbar = smem_u32(s_mbar + 1);
-  tc->cphase = 0;
 }
 
 __device__ inline void tc_teardown(TcState* tc) {

@@ -41,35 +41,41 @@ constexpr int kRfBits = 7;        // bits per slice
 constexpr int kRfSlicesA = 6;     // slices of A (42 bits)
 constexpr int kRfSlicesH = 4;     // slices of H' (28 bits)
 constexpr int kRfLevels = 6;      // products p + q = 0 .. 5 kept, one FP32 accumulator per level
-constexpr int kRfNMax = 80;       // columns of G per product tile: 64 or 80 per grid (rc.nN)
-constexpr int kRfKC = 32;         // K (contraction) extent of one staged chunk of the residual product
-constexpr int kRf2KC = 64;        // the same for the update product
-constexpr int kRfTileA = 128 * kRfKC * 2;        // bytes of one A slice of a (row block, K chunk)
-constexpr int kRfTileH = kRfNMax * kRfKC * 2;    // bytes of one H' slice of a (column block, K chunk)
-constexpr int kRfStage = kRfSlicesA * kRfTileA + kRfSlicesH * kRfTileH;  // 68 KiB: one chunk
-constexpr int kRfSmem = 2 * kRfStage;            // two stage buffers
+constexpr int kRfN = 64;          // rows of A per tile of the residual product (a tile: 128 columns of G)
+constexpr uint32_t kRfHead = 128; // bytes of parameters before the refinement's staging
+constexpr int kRf2KC = 32;        // K (contraction) extent of one staged chunk of the update product
 
 struct RefineConst {
-  const uint16_t* aslc;  // A's slices: [row block of 128][K chunk of 64][slice][128 x 64 FP16,
-                         // K-major core-matrix layout], padded with zeros
+  const uint16_t* tab;   // A's slices for sigma s_j = +1: [slice][block diagonal][8 x 8 FP16 core
+                         // matrix], block diagonal x = I + NJ - 1 - J for block row I, column J
   int ea;                // |A| < 2^ea (the slices' common scale)
-  int nrb, nkc;          // row blocks of 128, K chunks of 64 (Lambda padded)
   float emax_step;       // Newton steps only while max |E| <= emax_step (else from scratch)
-  int nN;                // columns of G per product tile: 64 or 80, whichever pads Lambda less
   float cplus[2];        // e^{+lambda}, e^{-lambda} in FP32: (1 + d_j) for sigma s_j = +1, -1
   float cminus_hi[2];    // e^{-sigma lambda s_j} = 1 / (1 + d_j) as an FP32 pair (hi + lo)
   float cminus_lo[2];
-  uint16_t dslc[2][kRfSlicesA];  // slices (FP16 bits) of A_jj for sigma s_j = +1, -1
+  float dd[kRfSlicesA];  // the diagonal's other value: the slices of A_jj for sigma s_j = -1,
+                         // less those for +1
 };
 
-__host__ __device__ inline int rf_pad(int L, int m) { return (L + m - 1) / m * m; }
-// Bytes of A's slice table of one grid, and of the per-chain workspace the
-// refinement needs (E^T in FP32, rows padded to a multiple of four floats;
-// the chain's FP64 Gauss-Jordan workspace has room).
-__host__ __device__ inline size_t rf_aslc_bytes(int L) {
-  return (size_t)(rf_pad(L, 128) / 128) * (rf_pad(L, kRfKC) / kRfKC) * kRfSlicesA * kRfTileA;
+__host__ __device__ constexpr int rf_pad(int L, int m) { return (L + m - 1) / m * m; }
+// Block rows of A (whole tiles of the residual product), block columns (the
+// contraction, padded to 16), and the block diagonals between them.
+__host__ __device__ constexpr int rf_ni(int L) { return rf_pad(L, kRfN) / 8; }
+__host__ __device__ constexpr int rf_nj(int L) { return rf_pad(L, 16) / 8; }
+__host__ __device__ constexpr int rf_ncore(int L) { return rf_ni(L) + rf_nj(L) - 1; }
+// Bytes of A's slice table of one grid (128 per core matrix), and of the
+// per-chain workspace the refinement needs: E in FP32, rows padded to a
+// multiple of eight floats, and with more than two column blocks of 128 the
+// new G beside it (the chain's FP64 Gauss-Jordan workspace has room).
+__host__ __device__ constexpr size_t rf_tab_bytes(int L) { return (size_t)kRfSlicesA * rf_ncore(L) * 128; }
+__host__ __device__ constexpr size_t rf_ws_bytes(int L) {
+  return (size_t)L * rf_pad(L, 8) * 4 + (L > 256 ? (size_t)L * L * 4 : 0);
 }
-__host__ __device__ inline size_t rf_ws_bytes(int L) { return (size_t)L * rf_pad(L, 4) * 4; }
+// One stage buffer of the update product: E^T hi and lo of one or two column
+// blocks of 128, H' hi and lo of every row.
+__host__ __device__ constexpr uint32_t rf_stage2_bytes(int L) {
+  return (uint32_t)((L > 128 && L <= 256 ? 2 : 1) * 128 + rf_pad(L, 16)) * kRf2KC * 4u;
+}
 
 struct GridConst {
   int L;           // Lambda

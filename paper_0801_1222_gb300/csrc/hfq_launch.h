@@ -25,7 +25,7 @@ inline cudaError_t raise_smem_limit(F* f, size_t smem) {
 int launch_bath_matrix(int L, const double* G0_tau, double* M, cudaStream_t st);
 int launch_bath_inverse(int L, const double* M, double* Minv, int* status, cudaStream_t st);
 // slices of A = M^{-1} - diag(...) for the Newton refinement of G (FP32 delayed path)
-int launch_refine_prep(int L, const double* Minv, double lambda, RefineConst* rc, uint16_t* aslc,
+int launch_refine_prep(int L, const double* Minv, double lambda, RefineConst* rc, uint16_t* tab,
                        cudaStream_t st);
 // initial (or refreshed) field and Green matrices of the chains of one grid
 int launch_init_chains(const SweepArgs& a, const GridConst* d_grid_ptr, int item0, int n_chains,

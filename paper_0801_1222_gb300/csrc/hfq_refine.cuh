@@ -16,25 +16,56 @@
 // cannot give; the residual product A H' is therefore formed from integer
 // slices (the splitting idea of Ozaki, Ogita, Oishi and Rump, written here
 // for FP16 tensor-core operands):
-//   * A (one table per grid, hfq_setup's k_refine_prep) = 2^ea sum_p a_p 2^{-7(p+1)},
-//     6 signed 7-bit slices; the field-dependent diagonal is patched in per chain;
+//   * A = 2^ea sum_p a_p 2^{-7(p+1)}, 6 signed 7-bit slices;
 //   * H' = the FP32 H = fl32((1 + d_j) G_jn) rounded to the grid 2^{eh-28}
-//     (eh: |H| < 2^eh) = 2^eh sum_q h_q 2^{-7(q+1)}, 4 slices, cut straight
-//     into shared memory chunk by chunk while A's slices arrive.  G' =
+//     (eh: |H| < 2^eh) = 2^eh sum_q h_q 2^{-7(q+1)}, 4 slices.  G' =
 //     (1 + D)^{-1} H' differs from G by at most half that grid step; E and
 //     the update both use this same G', so Newton's identity holds for it;
 //   * a_p, h_q are integers with |.| <= 128 (first slice) or <= 64, exact in
 //     FP16.  The products with p + q = l go to one FP32 TMEM accumulator per
 //     level l = 0..5 (at most four pairs, each K term <= 6 * 2^12 in all, so
 //     every partial sum is an integer below 2^24 for Lambda <= 512: the
-//     accumulation is exact).  Dropped levels and the slices' remainders
-//     leave |E - E_exact| ~ 1e-10 of |A||H'|.
-//   * The six level sums are combined exactly in 64-bit integers,
+//     accumulation is exact, in any order).  Dropped levels and the slices'
+//     remainders leave |E - E_exact| ~ 1e-10 of |A||H'|.
+//   * The six level sums are combined exactly in integers,
 //     V = sum_l S_l 2^{7 (5 - l)}, so A H' = V 2^{ea + eh - 49}, and
 //     E = delta - V 2^{ea+eh-49} is formed as an integer before it is
 //     rounded to FP32: the cancellation costs nothing.
+//
+// The residual product on the tensor cores, E^T = 1 - H'^T A^T tile by tile
+// (128 columns n of H' = TMEM lanes, 64 rows i of A):
+//   * M^{-1} is a function of i - j only (skew-circulant), so an 8 x 8 core
+//     matrix of A depends on the difference of its block row and block column
+//     alone: a slice needs one core matrix per block diagonal (2 L / 8, not
+//     L^2 / 64 of them), and the whole sliced A (45 KiB at Lambda = 240, 96
+//     at 512) stays in shared memory for the refinement.  With the
+//     contraction run through the blocks J in descending order the core of
+//     (I, J' = NJ - 1 - J) lies at (I + J') * 128 bytes: both descriptor
+//     strides are 128 bytes and neighbouring tiles overlap.  The earlier form
+//     streamed A's 48 KiB per 32 columns of the contraction from L2.
+//   * A_jj depends on the field.  The table carries the value for
+//     sigma s_j = +1; rows with sigma s_i = -1 get (A_ii difference) x H'_in
+//     added to V in the read-out, from the same slices of H'_in with the same
+//     products p + q <= 5 dropped, so V is the one of the sliced product.
+//   * H'^T is the other operand, cut from G by 15 warps straight into TMEM
+//     (the A operand of tcgen05.mma may live there): the tensor cores then
+//     read only A's slices, 2 KiB per MMA, from shared memory, and a 128 x 64
+//     x 16 MMA runs at its 32 cycles (measured alone: 32.1; with both operands
+//     in shared memory 48).  Four TMEM buffers of one K step of 16 each; the
+//     cutting warps and the issuing warp meet on mbarriers, there is no CTA
+//     barrier in the loop.
 // The update H' E only needs FP32 accuracy (|E| is small): split FP16
-// hi/lo parts with power-of-two scales, three products, FP32 accumulation.
+// hi/lo parts with power-of-two scales, three products, FP32 accumulation,
+// formed transposed as well (E^T H'^T) so that a warp's lanes are consecutive
+// columns of G in both read-outs and every access to G and E is coalesced.
+//
+// SM cycles per refinement of one spin at Lambda = 240 (phase timers in a copy
+// of the kernel), with A's slices streamed from L2 and H' cut into shared
+// memory, and as it is here: residual product 180k -> 132k (its MMAs alone
+// take 69k; what is above is the hand-over between the cutting warps and the
+// issuer, 50 cycles an MMA), its read-outs 50k -> 42k, update product 46k ->
+// 34k, its read-out 31k -> 26k, scale pass 16k -> 13k; at Lambda = 500 in all
+// 2.83M -> 1.98M.
 //
 // max |E| over the matrix decides: above rc.emax_step (2^-8 by default) the
 // step is not taken and the caller recomputes G from scratch (Gauss-Jordan);
@@ -50,25 +81,27 @@ namespace hfq {
 
 static_assert(kDelNT == 512, "the refinement's TMEM read-out assumes 16 warps");
 
-// The thread that issues (and commits) the residual product's MMAs: lane 0
-// of the last warp, which cuts no H' slices, so the issue overlaps the
-// slicing of the next chunk (threads 0 .. 255).
-constexpr int kRfIssuer = kDelNT - 32;
-static_assert(kRfIssuer >= kRfNMax * (kRfKC / 8), "the MMA issuer must not slice");
-static_assert(kTmemCols >= kRfLevels * kRfNMax, "level accumulators must fit the TMEM allocation");
+// TMEM columns of the residual product: kRfLevels accumulators of kRfN
+// columns, then kRfBufs buffers of H' slices (one K step of 16 each:
+// kRfSlicesH x 8 columns, two FP16 values of the contraction index per column)
+constexpr int kRfBufs = 4;
+constexpr int kRfBufCol = kRfLevels * kRfN;
+constexpr int kRfBufCols = kRfSlicesH * 8;
+static_assert(kRfBufCol + kRfBufs * kRfBufCols <= kTmemCols, "accumulators and H' buffers must fit the TMEM allocation");
+constexpr int kRfIssueWarp = 15;  // its elected lane issues every MMA; the other warps cut H'
+constexpr int kRfAhead = 2;       // K steps of the next tile cut before a tile's read-out
 
-// K-major core-matrix layout (8 rows x 16 bytes per core matrix, contiguous
-// along K): element (r, m) of a tile with K extent kRfKC (the residual
-// product's chunks) or kRf2KC (the update's)
-__device__ __forceinline__ uint32_t rf_off(int r, int m) {
-  return (uint32_t)((r >> 3) * (kRfKC / 8) * 128 + (m >> 3) * 128 + (r & 7) * 16 + (m & 7) * 2);
-}
-__device__ __forceinline__ uint32_t rf_off2(int r, int m) {
-  return (uint32_t)((r >> 3) * (kRf2KC / 8) * 128 + (m >> 3) * 128 + (r & 7) * 16 + (m & 7) * 2);
+// K-major core-matrix layout of the update product's chunks (8 rows x 16
+// bytes per core matrix, contiguous along K)
+__device__ __forceinline__ uint32_t rf_off2(int r, int k8) {
+  return (uint32_t)((r >> 3) * (kRf2KC / 8) * 128 + k8 * 128 + (r & 7) * 16);
 }
 
 __device__ __forceinline__ void mbar_expect_tx(uint32_t mbar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
 }
 
 // bulk copy global -> this CTA's shared memory, completion counted on mbar
@@ -79,21 +112,80 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
                : "memory");
 }
 
-__device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
-
 // 2^k as an FP32 number, -126 <= k <= 127 (scalings by it are exact while
 // the result stays normal)
 __device__ __forceinline__ float pow2f(int k) { return __int_as_float((127 + k) << 23); }
 
-// 32 lanes x 32 bit, 8 consecutive columns per thread
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
-  uint32_t r[8];
+// 32 lanes x 32 bit, 8 consecutive columns per thread; the values may be
+// used after tmem_wait_ld
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_ld4_nowait(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait_ld4(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])::"memory");
+}
+// the registers pass through the asm, so no use of them moves above the wait
+__device__ __forceinline__ void tmem_wait_ld8(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])::"memory");
+}
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(a), "r"(b), "r"(c),
+               "r"(d)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// One lane of the (converged) warp, as a predicate for the issuing lane: the
+// branch around the MMAs stays warp-uniform, so their descriptors live in
+// uniform registers (an issue from a divergent branch costs about 50 cycles).
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r;
+}
+// A warp-uniform value as one the compiler knows to be uniform (a warp
+// reduction's result is a uniform register; a shuffle's is not)
+__device__ __forceinline__ uint32_t rf_uniform(uint32_t x) { return __reduce_or_sync(0xffffffffu, x); }
+// kind::f16 MMA issued by the elected lane (el != 0), A operand in TMEM; the same lane's commit
+__device__ __forceinline__ void tc_mma_f16_ts(uint32_t el, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
+                                              uint32_t idesc, int accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "setp.ne.b32 e, %5, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      :
+      : "r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(el));
+}
+__device__ __forceinline__ void tc_commit_el(uint32_t el, uint32_t mbar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t"
+      "setp.ne.b32 e, %1, 0;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(mbar), "r"(el)
+      : "memory");
+}
+// kind::f16 MMA issued by the elected lane, both operands in shared memory
+__device__ __forceinline__ void tc_mma_f16_el(uint32_t el, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                              uint32_t idesc, int accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "setp.ne.b32 e, %5, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      :
+      : "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(el));
 }
 
 // Block-wide max of non-negative floats, NaN counted as infinity; every
@@ -111,451 +203,676 @@ __device__ __forceinline__ float rf_block_max(float v, float* red) {
   return r;
 }
 
-// x[0..7] = p[0..7], entries t >= n read as 0.  vec: p is 16-byte aligned
-// and n is a multiple of four (or <= 0), so two float4 loads serve.
-__device__ __forceinline__ void rf_ld8(const float* p, int n, bool vec, float* x) {
-  if (vec) {
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-    if (n >= 4) a = *reinterpret_cast<const float4*>(p);
-    if (n >= 8) b = *reinterpret_cast<const float4*>(p + 4);
-    x[0] = a.x, x[1] = a.y, x[2] = a.z, x[3] = a.w, x[4] = b.x, x[5] = b.y, x[6] = b.z, x[7] = b.w;
-  } else {
+// Eight values y (|y| < 2^7) -> four slices of 7 bits: slice q holds the
+// nearest integers (ties to even, as rintf) of the running remainders, which
+// then move up 7 bits; w[q]: slice q's eight FP16 values, packed.
+// Full-rate FP32 and FP16x2 arithmetic only: adding kC = 1.5 * 2^23 + 0x6600
+// rounds to an integer (the FP32 spacing there is 1, and kC is even, so ties
+// fall as they would without it) and leaves 0x6600 + v in the low 16 bits,
+// the FP16 number 1536 + v (spacing 1 in [1024, 2048)), of which 1536 is
+// subtracted exactly.  The remainder times 2^7 is two FMAs, exact as well.
+__device__ __forceinline__ void rf_cut8(float* y, uint32_t (*w)[4]) {
+  constexpr float kC = 12582912.f + 26112.f;
 #pragma unroll
-    for (int t = 0; t < 8; ++t) x[t] = t < n ? p[t] : 0.f;
+  for (int q = 0; q < kRfSlicesH; ++q) {
+#pragma unroll
+    for (int t = 0; t < 8; t += 2) {
+      const float ta = y[t] + kC, tb = y[t + 1] + kC;
+      const uint32_t pk = __byte_perm(__float_as_uint(ta), __float_as_uint(tb), 0x5410);
+      const uint32_t c1536 = 0x66006600u;
+      __half2 hv, hc;
+      memcpy(&hv, &pk, 4);
+      memcpy(&hc, &c1536, 4);
+      hv = __hsub2(hv, hc);
+      memcpy(&w[q][t / 2], &hv, 4);
+      if (q + 1 < kRfSlicesH) {
+        y[t] = __fmaf_rn(y[t], 128.f, __fmaf_rn(ta, -128.f, 128.f * kC));
+        y[t + 1] = __fmaf_rn(y[t + 1], 128.f, __fmaf_rn(tb, -128.f, 128.f * kC));
+      }
+    }
   }
 }
 
-// p[0..7] = x[0..7] for t < n (same vec contract as rf_ld8)
-__device__ __forceinline__ void rf_st8(float* p, int n, bool vec, const float* x) {
-  if (vec) {
-    if (n >= 4) *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
-    if (n >= 8) *reinterpret_cast<float4*>(p + 4) = make_float4(x[4], x[5], x[6], x[7]);
-  } else {
-#pragma unroll
-    for (int t = 0; t < 8; ++t)
-      if (t < n) p[t] = x[t];
+// One element of E = delta - V 2^{-sh} from its six level sums in 64-bit
+// integers, for |E| beyond the read-out's FP32 evaluation (see there).
+// taddr: the element's level-0 TMEM column; neg: its row has sigma s = -1, y
+// then being H'_in 2^{7-eh} and dd the diagonal's slice differences.
+__device__ __noinline__ float rf_residual_wide(uint32_t taddr, bool neg, float y, const float* dd, bool diag, int sh) {
+  float d[kRfSlicesH];
+  for (int q = 0; q < kRfSlicesH; ++q) {
+    d[q] = neg ? rintf(y) : 0.f;
+    y = (y - d[q]) * (float)(1 << kRfBits);
   }
+  long long V = 0;
+  for (int lv = 0; lv < kRfLevels; ++lv) {
+    uint32_t u;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(u) : "r"(taddr + (uint32_t)(lv * kRfN)));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(u)::"memory");
+    V = V * (1ll << kRfBits) + (long long)__float2int_rn(__uint_as_float(u));
+    for (int q = 0; q < kRfSlicesH && q <= lv; ++q) V += (long long)__float2int_rn(dd[lv - q] * d[q]);
+  }
+  const long long Ei = (diag ? 1ll << sh : 0ll) - V;
+  if (Ei > (1ll << 54) || Ei < -(1ll << 54)) return __int_as_float(0x7f800000);  // far beyond the step's range
+  const float hi = (float)(int)(Ei >> 24), lo = (float)(int)(Ei & 0xffffffll);
+  return fmaf(hi, 16777216.f, lo) * pow2f(-sh);
 }
 
-// The nearest integers ra, rb of a, b (|a|, |b| <= 2^7; ties to even, as
-// rintf) and both as FP16, packed (a in the low half), with full-rate FP32,
-// integer and FP16x2 arithmetic only: adding 1.5 * 2^23 rounds to an integer
-// (the FP32 spacing there is 1), whose bits give v; the FP16 bits of 1536 + v
-// are 0x6600 + v (spacing 1 in [1024, 2048)), and 1536 subtracted in FP16
-// leaves v exactly.
-__device__ __forceinline__ uint32_t rf_round_h2(float a, float b, float* ra, float* rb) {
-  const float ta = a + 12582912.f, tb = b + 12582912.f;
-  *ra = ta - 12582912.f;
-  *rb = tb - 12582912.f;
-  const uint32_t pk = ((0x6600u + (uint32_t)(__float_as_int(ta) - 0x4B400000)) & 0xffffu) |
-                      ((0x6600u + (uint32_t)(__float_as_int(tb) - 0x4B400000)) << 16);
-  const uint32_t c1536 = 0x66006600u;
-  __half2 hv, hc;
-  memcpy(&hv, &pk, 4);
-  memcpy(&hc, &c1536, 4);
-  hv = __hsub2(hv, hc);
-  uint32_t r;
-  memcpy(&r, &hv, 4);
-  return r;
+// What one refinement works with, at the start of its shared memory.  Each
+// phase takes its own copies of what it needs, so that little is live from
+// one phase to the next: with everything live throughout, the compiler spills
+// some hundred bytes per thread, which at 512 threads go to L2.
+struct RfPar {
+  float* G;
+  float* wsE;
+  const RefineConst* rc;
+  const int8_t* s;
+  int* status;
+  int L, ld, sig;
+  uint32_t tmem, cbar;
+  RfSync sync;
+};
+constexpr uint32_t kRfParBytes = 128;
+static_assert(sizeof(RfPar) <= kRfParBytes, "the parameters' slot in the refinement's shared memory");
+static_assert(kRfParBytes == kRfHead, "rf_smem_need counts the slot");
+
+__host__ __device__ constexpr int rf_lde(int L) { return rf_pad(L, 8); }
+
+// Bounded waits of one thread: after one has given up it waits no more
+struct RfWait {
+  bool bad = false;
+  __device__ __forceinline__ void on(uint32_t bar, uint32_t parity) {
+    if (!bad && !mbar_wait_bounded(bar, parity)) bad = true;
+  }
+};
+
+// The same for a whole (converged) warp, every branch on a vote: control flow
+// that the compiler knows to be uniform keeps the MMAs' operands in uniform
+// registers
+__device__ __forceinline__ bool rf_wait_warp(uint32_t mbar, uint32_t parity) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(mbar, parity))) return true;
+  const long long t0 = clock64();
+  while (!__all_sync(0xffffffffu, mbar_try_wait(mbar, parity)))
+    if (__any_sync(0xffffffffu, clock64() - t0 > (1ll << 31))) return false;
+  return true;
 }
 
-// One spin: G (L x L, row-major, FP32, in global memory) is replaced by its
-// Newton-refined value.  s: the field (shared memory); sig: +1 / -1; ws: the
-// chain's workspace (E^T: L rows of rf_pad(L, 4) floats); sm: rf_smem_need(L) of 1024-byte aligned
-// shared memory; tc: the CTA's TMEM allocation and mbarriers (tc->cbar: bulk
-// copies into the two stage buffers, then their MMA completions).
+// max |H|, H = fl32((1 + d_j) G_jn); NaN counts as infinity.  All threads.
+__device__ __forceinline__ float rf_scale(const RfPar& P, float* red) {
+  const int L = P.L, ld = P.ld, sig = P.sig;
+  const float* G = P.G;
+  const int8_t* s = P.s;
+  const float cpl0 = P.rc->cplus[0], cpl1 = P.rc->cplus[1];  // 1 + d_j for sigma s_j = +1, -1
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int NW = kDelNT / 32, RB = 4;  // rows per warp in flight, every load before its use
+  float hmax = 0.f;
+  for (int j0 = warp; j0 < L; j0 += RB * NW) {
+    for (int n0 = lane; n0 < L; n0 += 32 * 8) {
+      float g[RB][8];
+#pragma unroll
+      for (int r = 0; r < RB; ++r) {
+        const float* p = G + (size_t)min(j0 + r * NW, L - 1) * ld;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) g[r][u] = p[min(n0 + 32 * u, L - 1)];
+      }
+#pragma unroll
+      for (int r = 0; r < RB; ++r) {
+        const float cp = sig * s[min(j0 + r * NW, L - 1)] > 0 ? cpl0 : cpl1;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const float H = fabsf(g[r][u] * cp);
+          asm("max.NaN.f32 %0, %0, %1;" : "+f"(hmax) : "f"(H));  // a NaN enters and stays
+        }
+      }
+    }
+  }
+  return rf_block_max(hmax, red);
+}
+
+// E = 1 - A H' -> P.wsE (row stride rf_lde(L)), tile by tile (128 columns n of
+// H' = TMEM lanes, kRfN rows i of A); returns this thread's max |E|, sets
+// W.bad on a wait that gave up (then every thread returns early, together).
+// sm: A's table, then the row factors fs (zero beyond L).
+//
+// The cutting warps run through the contraction blocks of all tiles as one
+// stream (a quarter's blocks dealt round its warps), up to kRfAhead K steps
+// into the next tile before they turn to a tile's read-out.
+__device__ __forceinline__ float rf_product(RfPar& P, const unsigned char* sm, int sh, RfWait& W) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = (int)rf_uniform((uint32_t)tid >> 5);  // see elect_one
+  constexpr int NW = kDelNT / 32;
+  const int q4 = warp & 3, g4 = warp >> 2;  // TMEM lane quarter; group of rows or contraction blocks
+  const int L = P.L;
+  const int NJ = rf_nj(L), nib = rf_ni(L) / (kRfN / 8), nmb = (L + 127) / 128;
+  const uint32_t cc = P.sync.cc;
+  const uint32_t bar_full = P.cbar + 8u, bar_empty = bar_full + 8u * kRfBufs;
+  const uint32_t lane_base = P.tmem + ((uint32_t)(32 * q4) << 16);
+  const float* fs = reinterpret_cast<const float*>(sm + rf_tab_bytes(L));
+  const int stride = q4 == (kRfIssueWarp & 3) ? NW / 4 - 1 : NW / 4;
+  const int total = nmb * nib * NJ;
+  float emax = 0.f;
+  int vb = g4, vt = 0, vm = 0;  // the warp's next block: block of its tile, row tile, column block
+  int v = g4;                   // ... and its place in the stream
+  for (int tile = 0; tile < nmb * nib; ++tile) {
+    if (warp != kRfIssueWarp) {
+      // cut in registers, then stored once the buffer is free, so that little
+      // is left to do between a buffer's release and its refill; the loads of
+      // the warp's next block are issued before the cut.  A block: eight rows
+      // (in descending block order: see the table), one column per lane; lanes
+      // past the last column repeat it (their results are never read), rows
+      // past the last one count zero (fs is 0 there)
+      const int ld = P.ld;
+      const float* G = P.G;
+      float yn[8];  // the next block's values
+      auto load = [&]() {
+        const int j0 = 8 * (NJ - 1 - vb);
+        const float* p = G + min(vm * 128 + 32 * q4 + lane, L - 1);
+        if (j0 + 8 <= L) {
+          p += (size_t)j0 * ld;
+#pragma unroll
+          for (int t = 0; t < 8; ++t) {
+            yn[t] = *p;
+            p += ld;
+          }
+        } else {
+#pragma unroll
+          for (int t = 0; t < 8; ++t) yn[t] = p[(size_t)min(j0 + t, L - 1) * ld];
+        }
+      };
+      auto wrap = [&]() {
+        while (vb >= NJ) {
+          vb -= NJ;
+          if (++vt == nib) {
+            vt = 0;
+            ++vm;
+          }
+        }
+      };
+      const int lim = min((tile + 1) * NJ + 2 * kRfAhead, total);
+      wrap();
+      if (v < lim) load();
+#pragma unroll 1
+      while (v < lim) {
+        float y[8];
+        {
+          const float4* f4 = reinterpret_cast<const float4*>(fs + 8 * (NJ - 1 - vb));
+          const float4 f0 = f4[0], f1 = f4[1];
+          y[0] = yn[0] * f0.x, y[1] = yn[1] * f0.y, y[2] = yn[2] * f0.z, y[3] = yn[3] * f0.w;
+          y[4] = yn[4] * f1.x, y[5] = yn[5] * f1.y, y[6] = yn[6] * f1.z, y[7] = yn[7] * f1.w;
+        }
+        const int half = v & 1;  // NJ is even: also the block's half of its K step
+        const uint32_t nu = cc + (uint32_t)(v >> 1);
+        v += stride;
+        vb += stride;
+        wrap();
+        if (v < lim) load();
+        uint32_t w[kRfSlicesH][4];
+        rf_cut8(y, w);
+        if (nu >= kRfBufs) W.on(bar_empty + 8u * (nu % kRfBufs), (nu / kRfBufs - 1u) & 1u);
+        __syncwarp();
+        tc_fence_after();
+        const uint32_t col = lane_base + (uint32_t)(kRfBufCol + (int)(nu % kRfBufs) * kRfBufCols + half * 4);
+#pragma unroll
+        for (int q = 0; q < kRfSlicesH; ++q) tmem_st4(col + (uint32_t)(q * 8), w[q][0], w[q][1], w[q][2], w[q][3]);
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_full + 8u * (nu % kRfBufs));
+      }
+    } else {
+      // every operand of an MMA warp-uniform in the compiler's eyes
+      const uint32_t el = elect_one();
+      const uint32_t idesc = make_idesc_f16(kRfN);
+      const uint32_t n16 = (uint32_t)NJ / 2u, ib = (uint32_t)tile % (uint32_t)nib;
+      const uint32_t tm = rf_uniform(P.tmem), nk = rf_uniform(n16), bar_e = rf_uniform(bar_empty), bar_f = rf_uniform(bar_full);
+      const uint32_t c0 = rf_uniform(cc + (uint32_t)tile * n16), slice = rf_uniform((uint32_t)rf_ncore(L) * 8u);
+      const uint64_t desc = make_smem_desc(smem_u32(sm) + ib * (kRfN * 16u), 128u, 128u);
+      uint32_t bk = rf_uniform((uint32_t)desc);
+      bool live = !__any_sync(0xffffffffu, W.bad);
+      for (uint32_t k = 0; k < nk; ++k, bk += 16u) {
+        const uint32_t nu = c0 + k;
+        if (live) live = rf_wait_warp(bar_f + 8u * (nu % kRfBufs), (nu / kRfBufs) & 1u);
+        tc_fence_after();
+        const uint32_t a0 = tm + kRfBufCol + nu % kRfBufs * kRfBufCols;
+        const uint64_t bd = (desc & 0xffffffff00000000ull) | bk;
+        if (live) {
+#pragma unroll
+          for (int q = 0; q < kRfSlicesH; ++q)
+#pragma unroll
+            for (int p = 0; p + q < kRfLevels; ++p)
+              tc_mma_f16_ts(el, tm + (uint32_t)((p + q) * kRfN), a0 + (uint32_t)(q * 8), bd + (uint64_t)((uint32_t)p * slice),
+                            idesc, q > 0 || k > 0 ? 1 : 0);
+        }
+        tc_commit_el(el, bar_e + 8u * (nu % kRfBufs));
+      }
+      // the last step's products (the issuer has seen every use before it consumed)
+      const uint32_t nl = c0 + nk - 1u;
+      if (live) live = rf_wait_warp(bar_e + 8u * (nl % kRfBufs), (nl / kRfBufs) & 1u);
+      W.bad = !live;
+    }
+    // this warp's rows of the tile, ie .. ie + 15: those with sigma s = -1
+    // (whose diagonal differs from the table's), and G_in there, loaded while
+    // the last MMAs run
+    const int ie = tile % nib * kRfN + 16 * g4, n = tile / nib * 128 + 32 * q4 + lane;
+    const unsigned neg = __ballot_sync(
+        0xffffffffu, lane < 16 && ie + lane < L && P.sig * P.s[ie + lane < L ? ie + lane : 0] < 0);
+    float gd[16];
+    {
+      const float* p = P.G + (size_t)min(ie, L - 1) * P.ld + min(n, L - 1);
+      const int ld = P.ld;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        if (neg >> c & 1u) gd[c] = *p;  // warp-uniform
+        p += ld;
+      }
+    }
+    if (!__syncthreads_and(W.bad ? 0 : 1)) {
+      W.bad = true;
+      return emax;
+    }
+    tc_fence_after();
+    // Read-out, 4 rows at a time.  Horner's rule from the highest level,
+    // x <- 128 x + S_l, with delta subtracted at level 0, in FP32: where |E|
+    // is small the level sums cancel, every x up to level 4 is an integer
+    // below 2^24, so each FMA is exact and the last one rounds
+    // 2^{sh} (A H' - delta) once -- the same E as from 64-bit integers.
+    // Checked: an inexact x means |x_4| >= 2^24 (x only grows from there),
+    // and the warp evaluates those rows in 64 bits.
+    const bool narrow = sh >= 35;  // 2^{sh-35}, delta in units of level 0, is an integer
+    const float one0 = pow2f(narrow ? sh - 35 : 0), back = -pow2f(-sh);
+    float dd[kRfSlicesA];  // slices of A_jj for sigma s_j = -1 less those for +1
+#pragma unroll
+    for (int p = 0; p < kRfSlicesA; ++p) dd[p] = P.rc->dd[p];
+    float* pe = P.wsE + (size_t)ie * rf_lde(L) + n;
+    uint32_t widemask = 0u;  // rows to evaluate in 64 bits (warp-uniform)
+#pragma unroll
+    for (int h4 = 0; h4 < 4; ++h4) {
+      const int i0 = ie + 4 * h4;
+      if (i0 < L) {  // warp-uniform
+        const uint32_t ta = lane_base + (uint32_t)(16 * g4 + 4 * h4);
+        uint32_t u[kRfLevels][4];
+#pragma unroll
+        for (int lv = 0; lv < kRfLevels; ++lv) tmem_ld4_nowait(ta + (uint32_t)(lv * kRfN), u[lv]);
+        float x[4];
+#pragma unroll
+        for (int lv = 0; lv < kRfLevels; ++lv) tmem_wait_ld4(u[lv]);
+        bool wide = !narrow;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          float S[kRfLevels];
+#pragma unroll
+          for (int lv = 0; lv < kRfLevels; ++lv) S[lv] = __uint_as_float(u[lv][c]);
+          if (neg >> (4 * h4 + c) & 1u) {  // warp-uniform: the other value of A_ii
+            float y = gd[4 * h4 + c] * fs[i0 + c];
+#pragma unroll
+            for (int q = 0; q < kRfSlicesH; ++q) {
+              const float d = (y + 12582912.f) - 12582912.f;
+#pragma unroll
+              for (int p = 0; p + q < kRfLevels; ++p) S[p + q] = __fmaf_rn(dd[p], d, S[p + q]);
+              y = __fmaf_rn(y, 128.f, -128.f * d);
+            }
+          }
+          x[c] = S[0] - (i0 + c == n ? one0 : 0.f);
+#pragma unroll
+          for (int lv = 1; lv < kRfLevels; ++lv) {
+            if (lv == kRfLevels - 1) wide = wide || !(fabsf(x[c]) < 16777216.f);
+            x[c] = __fmaf_rn(x[c], 128.f, S[lv]);
+          }
+          x[c] = __fmaf_rn(x[c], back, 0.f);  // E (and +0 for a zero)
+        }
+        if (__any_sync(0xffffffffu, wide && n < L)) {
+          widemask |= 15u << (4 * h4);
+        } else if (n < L) {
+          // every value before the first store (which would order the loads after it)
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (i0 + c < L) {
+              pe[(size_t)(4 * h4 + c) * rf_lde(L)] = x[c];
+              emax = fmaxf(emax, fabsf(x[c]));
+            }
+        }
+      }
+    }
+#pragma unroll 1
+    for (; widemask; widemask &= widemask - 1u) {  // warp-uniform
+      const int c = __ffs(widemask) - 1, i = ie + c;
+      if (i >= L) break;
+      const bool ng = neg >> c & 1u;
+      const float y = ng ? P.G[(size_t)i * P.ld + min(n, L - 1)] * fs[i] : 0.f;
+      const float E = rf_residual_wide(lane_base + (uint32_t)(16 * g4 + c), ng, y, P.rc->dd, i == n, sh);
+      if (n < L) {
+        P.wsE[(size_t)i * rf_lde(L) + n] = E;
+        emax = fmaxf(emax, fabsf(E));
+      }
+    }
+    tc_fence_before();
+    __syncthreads();
+  }
+  if (tid == 0) P.sync.cc = cc + (uint32_t)(nmb * nib) * (uint32_t)(NJ / 2);
+  return emax;
+}
+
+// G_new^T = (H'^T + E^T H'^T) (1 + D)^{-1}, G replaced; returns this thread's
+// largest change of an entry, W.bad as above.  M: columns n of G (E^T), in
+// blocks of 128; N: all rows i (H'), up to 256 per MMA; K in chunks of kRf2KC
+// through two stage buffers (sm): a chunk is staged while the tensor cores
+// multiply the one before.
+__device__ __forceinline__ float rf_update(RfPar& P, unsigned char* sm, int eh, int se, RfWait& W) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = (int)rf_uniform((uint32_t)tid >> 5);
+  constexpr int NW = kDelNT / 32;
+  const int q4 = warp & 3, g4 = warp >> 2;
+  const int L = P.L, ld = P.ld, ldE = rf_lde(L), nmb = (L + 127) / 128;
+  float* const G = P.G;
+  const float* const wsE = P.wsE;
+  const int Lp = rf_pad(L, 16), nkc2 = rf_pad(L, kRf2KC) / kRf2KC;
+  // two column blocks and at most 256 rows: both blocks' products at once
+  // (accumulators at TMEM columns 0 and 256), so each H' chunk is staged once;
+  // else one column block at a time, its rows in up to two halves
+  const int nr = (nmb == 2 && Lp <= 256) ? 2 : 1;
+  const bool direct = nmb <= nr;  // every column block done before G is written
+  const bool vec = (ld & 3) == 0;  // rows of G 16-byte aligned
+  const uint32_t ebytes = 128u * kRf2KC * 2u;          // one column block's E^T hi (or lo)
+  const uint32_t hbytes = (uint32_t)Lp * kRf2KC * 2u;  // H' hi (or lo)
+  const uint32_t stage_bytes = rf_stage2_bytes(L), bar_stage = P.cbar + 8u + 16u * kRfBufs;
+  uint32_t c2 = P.sync.c2;
+  float drift = 0.f;
+  // per row: (1 + d_i) 2^{28-eh} (H' = rint(H 2^{28-eh}) 2^{eh-28}) and the FP32 pair of 1 / (1 + d_i)
+  float4* const rf = reinterpret_cast<float4*>(sm + 2 * stage_bytes);
+  for (int i = tid; i < Lp; i += kDelNT) {
+    const int u = i < L && P.sig * P.s[i < L ? i : 0] > 0 ? 0 : 1;
+    rf[i] = make_float4(P.rc->cplus[u] * pow2f(28 - eh), P.rc->cminus_hi[u], P.rc->cminus_lo[u], 0.f);
+  }
+  __syncthreads();
+  for (int mb0 = 0; mb0 < nmb; mb0 += nr) {
+    {
+      // E^T: thread = column n (lanes consecutive: coalesced), 8 rows j.  H':
+      // chunk c = row 8 (c / 32) + c % 8, K offset 8 ((c / 8) % 4): a warp
+      // covers 8 rows x 32 consecutive columns.  The loads of the next chunk
+      // are issued before the barrier of the current one
+      const float sE = pow2f(se);
+      const int k8e = tid >> 7, re = tid & 127;
+      float xe[2][8], xh[2][8];
+      auto load_e = [&](int kc) {
+        const int j0 = kc * kRf2KC + 8 * k8e;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          if (u < nr) {
+            // columns past the last repeat it (never read back); rows past it are 0
+            const float* p = wsE + (size_t)j0 * ldE + min((mb0 + u) * 128 + re, L - 1);
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+              xe[u][t] = j0 + t < L ? *p : 0.f;
+              p += ldE;
+            }
+          }
+        }
+      };
+      auto load_h = [&](int kc, int c0) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int c = c0 + u * kDelNT, i = min(((c >> 5) << 3) | (c & 7), L - 1);
+          const int k0 = kc * kRf2KC + (((c >> 3) & 3) << 3);
+          const float* p = G + (size_t)i * ld + k0;
+          if (vec && k0 + 8 <= L) {
+            const float4 x0 = *reinterpret_cast<const float4*>(p), x1 = *reinterpret_cast<const float4*>(p + 4);
+            xh[u][0] = x0.x, xh[u][1] = x0.y, xh[u][2] = x0.z, xh[u][3] = x0.w;
+            xh[u][4] = x1.x, xh[u][5] = x1.y, xh[u][6] = x1.z, xh[u][7] = x1.w;
+          } else {
+#pragma unroll
+            for (int t = 0; t < 8; ++t) xh[u][t] = k0 + t < L ? p[t] : 0.f;
+          }
+        }
+      };
+      load_e(0);
+      load_h(0, tid);
+      for (int kc = 0; kc < nkc2; ++kc, ++c2) {
+        if (c2 >= 2u) W.on(bar_stage + 8u * (c2 & 1u), ((c2 >> 1) - 1u) & 1u);
+        unsigned char* sb = sm + (c2 & 1u) * stage_bytes;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          if (u < nr) {
+            uint32_t h[4], l[4];
+#pragma unroll
+            for (int t = 0; t < 8; t += 2) {
+              const float xa = xe[u][t] * sE, xb = xe[u][t + 1] * sE;
+              h[t / 2] = f32x2_to_f16x2(xa, xb);
+              l[t / 2] = f32x2_to_f16x2(xa - f16_lo_to_f32(h[t / 2]), xb - f16_hi_to_f32(h[t / 2]));
+            }
+            unsigned char* dst = sb + u * 2 * ebytes + rf_off2(re, k8e);
+            *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<uint4*>(dst + ebytes) = make_uint4(l[0], l[1], l[2], l[3]);
+          }
+        }
+        if (kc + 1 < nkc2) load_e(kc + 1);
+        // H' (x 2^{14-eh}, below 2^14)
+        for (int c0 = tid;;) {
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int c = c0 + u * kDelNT, i = ((c >> 5) << 3) | (c & 7);
+            if (c < Lp * 4) {
+              const float cs = rf[i].x;
+              uint32_t h[4], l[4];
+#pragma unroll
+              for (int t = 0; t < 8; t += 2) {
+                const float xa = rintf(xh[u][t] * cs) * 0x1p-14f, xb = rintf(xh[u][t + 1] * cs) * 0x1p-14f;
+                h[t / 2] = f32x2_to_f16x2(xa, xb);
+                l[t / 2] = f32x2_to_f16x2(xa - f16_lo_to_f32(h[t / 2]), xb - f16_hi_to_f32(h[t / 2]));
+              }
+              unsigned char* dst = sb + nr * 2 * ebytes + rf_off2(i, (c >> 3) & 3);
+              *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
+              *reinterpret_cast<uint4*>(dst + hbytes) = make_uint4(l[0], l[1], l[2], l[3]);
+            }
+          }
+          c0 += 2 * kDelNT;
+          if (c0 >= Lp * 4) break;  // more than 256 rows: a second part, not prefetched
+          load_h(kc, c0);
+        }
+        if (kc + 1 < nkc2) load_h(kc + 1, tid);
+        fence_async_smem();
+        tc_fence_before();
+        if (!__syncthreads_and(W.bad ? 0 : 1)) {
+          W.bad = true;
+          return drift;
+        }
+        if (warp == kRfIssueWarp) {
+          tc_fence_after();
+          const uint32_t el = elect_one();
+          const uint32_t tm = rf_uniform(P.tmem), nru = rf_uniform((uint32_t)nr), lpu = rf_uniform((uint32_t)Lp);
+          const uint32_t e2 = rf_uniform(smem_u32(sb)), h2 = e2 + nru * 2u * ebytes;
+          const uint32_t kcu = rf_uniform((uint32_t)kc);
+          const uint64_t lo_e = (uint64_t)(ebytes >> 4), lo_h = (uint64_t)(lpu * (kRf2KC * 2u) >> 4);
+          const uint64_t ed = make_smem_desc(e2, 128u, (kRf2KC / 8) * 128u);
+          const uint64_t hd = make_smem_desc(h2, 128u, (kRf2KC / 8) * 128u);
+          for (uint32_t ur = 0; ur < nru; ++ur)
+            for (uint32_t half = 0; half * 256 < lpu; ++half) {
+              const uint32_t idesc2 = make_idesc_f16((int)min(lpu - half * 256u, 256u));
+              const uint32_t d = tm + (ur + half) * 256u;
+#pragma unroll
+              for (uint32_t kk = 0; kk < kRf2KC / 16; ++kk) {
+                if (kcu * kRf2KC + kk * 16 >= lpu) continue;
+                const uint64_t ahi = ed + (uint64_t)(ur * (2u * ebytes >> 4) + kk * 16u);
+                const uint64_t bhi = hd + (uint64_t)(half * (32u * (kRf2KC / 8) * 8u) + kk * 16u);
+                tc_mma_f16_el(el, d, ahi, bhi, idesc2, (kcu > 0 || kk > 0) ? 1 : 0);
+                tc_mma_f16_el(el, d, ahi + lo_e, bhi, idesc2, 1);
+                tc_mma_f16_el(el, d, ahi, bhi + lo_h, idesc2, 1);
+              }
+            }
+          if (el) tc_commit(bar_stage + 8u * (c2 & 1u));
+          __syncwarp();
+        }
+      }
+    }
+    // every product of this group of column blocks
+    W.on(bar_stage + 8u * ((c2 - 1u) & 1u), ((c2 - 1u) >> 1) & 1u);
+    if (!__syncthreads_and(W.bad ? 0 : 1)) {
+      W.bad = true;
+      return drift;
+    }
+    tc_fence_after();
+    // read-out: thread = column n, 8 rows i per pass (32 rows of the four
+    // groups of warps); the next pass's loads of G are issued before the
+    // current pass's arithmetic, the stores come last (a store in between
+    // would hold back the loads after it)
+    {
+      const float sHi = pow2f(eh - 28), sQ = pow2f(eh - 14 - se);
+      const uint32_t lane_base = P.tmem + ((uint32_t)(32 * q4) << 16);
+      float* const Gn = direct ? G : P.wsE + (size_t)L * ldE;
+      const int ldn = direct ? ld : L;
+#pragma unroll 1
+      for (int ur = 0; ur < nr; ++ur) {
+        const int n = (mb0 + ur) * 128 + 32 * q4 + lane;
+        float go[8];
+        auto load_g = [&](int i0) {
+          const float* p = G + (size_t)i0 * ld + min(n, L - 1);
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            if (i0 + c < L) go[c] = *p;  // warp-uniform
+            p += ld;
+          }
+        };
+        load_g(8 * g4);
+#pragma unroll 1
+        for (int i0 = 8 * g4; i0 < L; i0 += 32) {
+          float g[8];
+          uint32_t q[8];
+#pragma unroll
+          for (int c = 0; c < 8; ++c) g[c] = go[c];
+          load_g(i0 + 32);
+          tmem_ld8_nowait(lane_base + (uint32_t)(256 * ur + i0), q);
+          tmem_wait_ld8(q);
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            const float4 f = rf[min(i0 + c, Lp - 1)];
+            const float Hp = rintf(g[c] * f.x) * sHi;
+            const float y = Hp + __uint_as_float(q[c]) * sQ;
+            q[c] = __float_as_uint(fmaf(y, f.y, y * f.z));
+          }
+          if (n < L) {
+            float* p = Gn + (size_t)i0 * ldn + n;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              if (i0 + c < L) {  // warp-uniform
+                const float gn = __uint_as_float(q[c]);
+                drift = fmaxf(drift, fabsf(g[c] - gn));
+                *p = gn;
+              }
+              p += ldn;
+            }
+          }
+        }
+      }
+    }
+    tc_fence_before();
+    __syncthreads();
+  }
+  if (!direct) {
+    // every column block has read the old G: the new one moves in
+    const float* Gn = wsE + (size_t)L * ldE;
+    for (int i0 = warp; i0 < L; i0 += 2 * NW)
+      for (int n0 = lane; n0 < L; n0 += 32 * 8) {
+        float x[2][8];
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            x[r][u] = (i0 + r * NW < L && n0 + 32 * u < L) ? Gn[(size_t)(i0 + r * NW) * L + n0 + 32 * u] : 0.f;
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (i0 + r * NW < L && n0 + 32 * u < L) G[(size_t)(i0 + r * NW) * ld + n0 + 32 * u] = x[r][u];
+      }
+    __syncthreads();
+  }
+  if (tid == 0) P.sync.c2 = c2;
+  return drift;
+}
+
+// One spin: G (L x L, row-major, row stride ld, FP32, in global memory or in
+// shared memory outside sm) is replaced by its Newton-refined value.  s: the
+// field (shared memory); sig: +1 / -1; ws: the chain's workspace
+// (rf_ws_bytes: E, and beyond 256 columns the new G); sm0: rf_smem_need(L) of
+// 1024-byte aligned shared memory; tc: the CTA's TMEM allocation and
+// mbarriers (tc->cbar: table copy, the H' buffers' "full", their "empty", the
+// two update stages' "empty"; sync, in shared memory, counts their uses).
 // Returns the largest change of an entry (>= 0), or -1 if the caller must
 // recompute from scratch (|E| too large, scale out of range, or a wait gave
 // up, which also sets kStatusTimeout).  All threads call it.
-__device__ inline float refine_spin(const GridConst& gc, const RefineConst& rc, const int8_t* s, int sig,
-                                    float* G, float* ws, unsigned char* sm, TcState* tc, float* red, int* status,
-                                    int* steps) {
-  const int L = gc.L;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int NW = kDelNT / 32;
-  const int q4 = warp & 3, g4 = warp >> 2;  // TMEM lane quarter, column group (the update's epilogue)
-  const int nkc = rc.nkc, nrb = rc.nrb;
-  const int nN = rc.nN, nnb = rf_pad(L, nN) / nN;
-  float* wsE = ws;
-  const int ldE = rf_pad(L, 4);     // row stride of E^T in ws
-  const bool vec = (L & 3) == 0;    // rows of G 16-byte aligned: float4 accesses
-  const uint32_t sm0 = smem_u32(sm);
-  // the row factors in registers: (1 + d_j) and its inverse as an FP32 pair,
-  // selected by sigma s_j (index 0: +1, 1: -1)
-  const float cpl0 = rc.cplus[0], cpl1 = rc.cplus[1];
-  const float cmh0 = rc.cminus_hi[0], cmh1 = rc.cminus_hi[1], cml0 = rc.cminus_lo[0], cml1 = rc.cminus_lo[1];
-  float drift = 0.f;
-  uint32_t ph = tc->cphase;  // parity bits of the four barriers: copy 0, copy 1, MMA 0, MMA 1
-  for (int step = 0; step < 2; ++step) {
-    // ---- H = (1 + d_j) G_jn: its scale ------------------------------------
-    float hmax = 0.f;
-    for (int j = warp; j < L; j += NW) {
-      const float cp = sig * s[j] > 0 ? cpl0 : cpl1;
-      const float* Gj = G + (size_t)j * L;
-      for (int n0 = 0; n0 < L; n0 += 32 * 8) {
-        float g[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) g[u] = (n0 + 32 * u + lane < L) ? Gj[n0 + 32 * u + lane] : 0.f;  // loads first
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const float H = g[u] * cp;
-          hmax = (H == H) ? fmaxf(hmax, fabsf(H)) : __int_as_float(0x7f800000);
-        }
-      }
+__device__ __forceinline__ float refine_spin(const GridConst& gc, const RefineConst* rc, const int8_t* s, int sig,
+                                             float* G, int ld, float* ws, unsigned char* sm0, TcState* tc,
+                                             RfSync* sync, float* red, int* status) {
+  RfPar& P = *reinterpret_cast<RfPar*>(sm0);
+  unsigned char* sm = sm0 + kRfParBytes;
+  // what the region held before was read and written through the generic proxy
+  fence_async_smem();
+  __syncthreads();
+  if (threadIdx.x == 0) P = RfPar{G, ws, rc, s, status, gc.L, ld, sig, tc->tmem, tc->cbar, *sync};
+  __syncthreads();
+  RfWait W;
+  float drift = 0.f, emax = 0.f;
+  bool ok = true;
+  for (int step = 0; step < 2 && ok; ++step) {
+    // A's slice table into shared memory while the scale pass runs
+    if (threadIdx.x == 0) {
+      const uint32_t bytes = (uint32_t)rf_tab_bytes(P.L);
+      mbar_expect_tx(P.cbar, bytes);
+      bulk_g2s(smem_u32(sm), P.rc->tab, bytes, P.cbar);
     }
-    hmax = rf_block_max(hmax, red);
+    const float hmax = rf_scale(P, red);
+    W.on(P.cbar, P.sync.ct & 1u);
     int eh = 0;
-    if (!(hmax < 1e30f)) {
-      tc->cphase = ph;
-      return -1.f;
+    ok = hmax < 1e30f;
+    if (ok && hmax > 0.f) (void)frexpf(hmax, &eh);  // hmax < 2^eh
+    const int sh = 49 - P.rc->ea - eh;              // delta in units of the integer sums
+    ok = ok && !(sh < 0 || sh > 61 || eh < -60 || eh > 100);  // keeps every scale below normal
+    {
+      // (1 + d_j) 2^{7-eh}: H 2^{7-eh} is below 2^7 in magnitude
+      const int L = P.L;
+      const float s7 = pow2f(ok ? kRfBits - eh : 0);
+      float* fs = reinterpret_cast<float*>(sm + rf_tab_bytes(L));
+      for (int j = threadIdx.x; j < 8 * rf_nj(L); j += kDelNT)
+        fs[j] = j < L ? P.rc->cplus[P.sig * P.s[j] > 0 ? 0 : 1] * s7 : 0.f;
     }
-    if (hmax > 0.f) (void)frexpf(hmax, &eh);  // hmax < 2^eh
-    const int sh = 49 - rc.ea - eh;           // delta in units of the integer sums
-    if (sh < 0 || sh > 61 || eh < -60 || eh > 100) {  // keeps every scale below normal
-      tc->cphase = ph;
-      return -1.f;
+    __syncthreads();
+    if (threadIdx.x == 0) ++P.sync.ct;
+    if (!__syncthreads_and(W.bad ? 0 : 1)) {
+      W.bad = true;
+      break;
     }
-    const float s7 = pow2f(kRfBits - eh);  // H 2^{7-eh}: below 2^7 in magnitude
-
-    // ---- GEMM1: E = 1 - A H', tile by tile (128 rows x nN columns) ---------
-    // K goes in chunks of 32 through two stage buffers (A's six slices, 48
-    // KiB, by one bulk copy; H''s four, up to 20 KiB, cut by nN * 4 threads from G):
-    // chunk kc + 1 is brought in while the tensor cores multiply chunk kc.
-    // Every commit of a chunk's MMAs is waited for exactly once, in order,
-    // so each barrier's parity stays in step.
-    float emax = 0.f;
-    const uint32_t idesc1 = make_idesc_f16(nN);
-    bool bad = false;  // a bounded wait gave up
-    auto stage_in = [&](int nb, int rb, int kc, int b) {
-      const uint32_t bar = tc->cbar + 8u * (uint32_t)b;
-      if (tid == 0) {
-        mbar_expect_tx(bar, (uint32_t)(kRfSlicesA * kRfTileA));
-        bulk_g2s(sm0 + (uint32_t)(b * kRfStage), rc.aslc + (size_t)(rb * nkc + kc) * kRfSlicesA * (kRfTileA / 2),
-                 (uint32_t)(kRfSlicesA * kRfTileA), bar);
-      }
-      if (tid < nN * (kRfKC / 8)) {
-        // a column and eight rows of H' per thread, sliced into the buffer
-        const int j8 = tid / nN, nl = tid - j8 * nN;
-        const int n = nb * nN + nl, j0 = kc * kRfKC + j8 * 8;
-        float y[8];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          const int j = j0 + t;
-          y[t] = (j < L && n < L) ? G[(size_t)j * L + n] : 0.f;  // all loads first
-        }
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          const int j = j0 + t;
-          y[t] = y[t] * (j < L && sig * s[j] > 0 ? cpl0 : cpl1) * s7;
-        }
-        unsigned char* dst = sm + b * kRfStage + kRfSlicesA * kRfTileA + rf_off(nl, j8 * 8);
-#pragma unroll
-        for (int q = 0; q < kRfSlicesH; ++q) {
-          // slice q: the nearest integer v of the running remainder (below
-          // 2^7 in magnitude), which then moves up 7 bits
-          uint32_t w[4];
-#pragma unroll
-          for (int t = 0; t < 8; t += 2) {
-            float ra, rb2;
-            w[t / 2] = rf_round_h2(y[t], y[t + 1], &ra, &rb2);
-            y[t] = (y[t] - ra) * (float)(1 << kRfBits);
-            y[t + 1] = (y[t + 1] - rb2) * (float)(1 << kRfBits);
-          }
-          *reinterpret_cast<uint4*>(dst + q * kRfTileH) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-      }
-    };
-    auto wait_mma = [&](int b) {  // chunk MMAs of buffer b complete (every thread)
-      const uint32_t bit = 4u << b;
-      if (!mbar_wait_bounded(tc->cbar + 16u + 8u * (uint32_t)b, (ph & bit) ? 1u : 0u)) bad = true;
-      ph ^= bit;
-    };
-    for (int nb = 0; nb < nnb; ++nb) {
-      for (int rb = 0; rb < nrb; ++rb) {
-        stage_in(nb, rb, 0, 0);
-        for (int kc = 0; kc < nkc; ++kc) {
-          const int b = kc & 1;
-          const uint32_t cbit = 1u << b;
-          const bool got = mbar_wait_bounded(tc->cbar + 8u * (uint32_t)b, (ph & cbit) ? 1u : 0u);
-          ph ^= cbit;
-          // the field-dependent diagonal of A
-          if (tid < kRfKC) {
-            const int j = kc * kRfKC + tid;
-            if (j >= rb * 128 && j < rb * 128 + 128 && j < L) {
-              const int v = sig * s[j] > 0 ? 0 : 1;
-              const uint32_t off = rf_off(j - rb * 128, tid);
-#pragma unroll
-              for (int p = 0; p < kRfSlicesA; ++p)
-                *reinterpret_cast<uint16_t*>(sm + b * kRfStage + p * kRfTileA + off) = rc.dslc[v][p];
-            }
-          }
-          fence_async_smem();
-          tc_fence_before();
-          if (!__syncthreads_and((got && !bad) ? 1 : 0)) {
-            if (tid == 0) atomicOr(status, kStatusTimeout);
-            tc->failed = 1;
-            tc->cphase = ph;
-            return -1.f;
-          }
-          if (tid == kRfIssuer) {
-            tc_fence_after();
-            // descriptors of slice p / q at K step kk: the base one plus the
-            // byte offset >> 4 in the start-address field (no carry out of it:
-            // shared addresses stay below 256 KiB); the first product of a
-            // level in a tile starts its accumulator
-            const uint32_t aB = sm0 + (uint32_t)(b * kRfStage), hB = aB + (uint32_t)(kRfSlicesA * kRfTileA);
-#pragma unroll
-            for (int kk = 0; kk < kRfKC / 16; ++kk) {
-              const uint64_t da = make_smem_desc(aB + (uint32_t)(kk * 256), 128u, (kRfKC / 8) * 128u);
-              const uint64_t db = make_smem_desc(hB + (uint32_t)(kk * 256), 128u, (kRfKC / 8) * 128u);
-#pragma unroll
-              for (int p = 0; p < kRfSlicesA; ++p)
-#pragma unroll
-                for (int q = 0; q < kRfSlicesH; ++q) {
-                  const int lv = p + q;
-                  if (lv >= kRfLevels) continue;
-                  const int first_p = lv > kRfSlicesH - 1 ? lv - (kRfSlicesH - 1) : 0;
-                  const int acc = (kc > 0 || kk > 0 || p != first_p) ? 1 : 0;
-                  tc_mma_f16(tc->tmem + (uint32_t)(lv * nN), da + (uint64_t)(p * (kRfTileA >> 4)),
-                             db + (uint64_t)(q * (kRfTileH >> 4)), idesc1, acc);
-                }
-            }
-            tc_commit(tc->cbar + 16u + 8u * (uint32_t)b);
-          }
-          if (kc >= 1) wait_mma(b ^ 1);  // chunk kc - 1 done: its buffer is free
-          if (kc + 1 < nkc) stage_in(nb, rb, kc + 1, b ^ 1);
-        }
-        wait_mma((nkc - 1) & 1);
-        if (!__syncthreads_and(bad ? 0 : 1)) {
-          if (tid == 0) atomicOr(status, kStatusTimeout);
-          tc->failed = 1;
-          tc->cphase = ph;
-          return -1.f;
-        }
-        tc_fence_after();
-        // the six level sums of a row and 16 columns per task (TMEM lane
-        // quarter warp % 4, columns 16 g ..), 8 at a time, combined in 64-bit
-        // integers, then E = delta - V 2^{ea+eh-49}
-        const long long one = 1ll << sh;
-#pragma unroll 1
-        for (int task = warp; task < 4 * (nN / 16); task += NW) {
-          const int g16 = task >> 2;
-          const int i = rb * 128 + 32 * q4 + lane;
-#pragma unroll 1
-          for (int h8 = 0; h8 < 2; ++h8) {
-            long long V[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) V[c] = 0;
-#pragma unroll
-            for (int lv = 0; lv < kRfLevels; ++lv) {
-              float v[8];
-              tmem_ld8(tc->tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(lv * nN + 16 * g16 + 8 * h8), v);
-#pragma unroll
-              for (int c = 0; c < 8; ++c) V[c] = V[c] * (1ll << kRfBits) + (long long)__float2int_rn(v[c]);
-            }
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              const int n = nb * nN + 16 * g16 + 8 * h8 + c;
-              const long long Ei = (i == n ? one : 0ll) - V[c];
-              float E;
-              if (Ei > (1ll << 54) || Ei < -(1ll << 54)) {
-                E = __int_as_float(0x7f800000);  // far beyond the step's range
-              } else {
-                const float hi = (float)(int)(Ei >> 24), lo = (float)(int)(Ei & 0xffffffll);
-                E = fmaf(hi, 16777216.f, lo) * pow2f(-sh);
-              }
-              // E^T: lanes (rows i) write consecutive words; rows i >= L of E
-              // are exactly 0 (A's table is zero there), which fills the
-              // padding of E^T's rows
-              if (i < ldE && n < L) wsE[(size_t)n * ldE + i] = E;
-              if (i < L && n < L) emax = fmaxf(emax, fabsf(E));
-            }
-          }
-        }
-        tc_fence_before();
-        __syncthreads();
-      }
-    }
+    if (!ok) break;
+    emax = rf_product(P, sm, sh, W);
+    if (W.bad) break;
     emax = rf_block_max(emax, red);
-    if (!(emax <= rc.emax_step)) {  // too far for Newton steps (default 2^-8)
-      tc->cphase = ph;
-      return -1.f;
-    }
+    ok = emax <= P.rc->emax_step;  // else too far for Newton steps (default 2^-8)
+    if (!ok) break;
     int ee = 0;
     if (emax > 0.f) (void)frexpf(emax, &ee);  // emax < 2^ee
     // E 2^se below 2^15 (FP16 range); for |E| < 2^-25 the scale stops at
     // 2^40, where those corrections are far below G's FP32 rounding anyway
     const int se = emax > 0.f ? min(15 - ee, 40) : 0;
-
-    // ---- GEMM2: G_new = (1 + D)^{-1} (H' + H' E), 128 rows x all columns ----
-    const int Lp = rf_pad(L, 16), nkc2 = rf_pad(L, kRf2KC) / kRf2KC;
-    const uint32_t bl = (uint32_t)Lp * kRf2KC * 2u;  // bytes of one E^T part (hi or lo)
-    constexpr uint32_t kAbuf = 2u * 128u * kRf2KC * 2u;  // one row block's H' hi and lo
-    const float sH = pow2f(28 - eh);                // H' = rint(H 2^{28-eh}) 2^{eh-28}
-    const float sE = pow2f(se), sHi = pow2f(eh - 28), sQ = pow2f(eh - 14 - se);
-    // two row blocks of 128 and at most 256 columns: both blocks' products at
-    // once (accumulators at TMEM columns 0 and 256), so each E^T chunk is
-    // staged once; else one row block at a time
-    const int nr = (nrb == 2 && Lp <= 256) ? 2 : 1;
-    const uint32_t b2 = sm0 + (uint32_t)nr * kAbuf;
-    for (int rb0 = 0; rb0 < nrb; rb0 += nr) {
-      for (int kc = 0; kc < nkc2; ++kc) {
-#pragma unroll 1
-        for (int ur = 0; ur < nr; ++ur) {
-        const int rb = rb0 + ur;
-        unsigned char* sa = sm + ur * kAbuf;
-        // A: H' of rows rb*128.. (x 2^{14-eh}, below 2^14), hi / lo: 1024
-        // chunks of eight K values, two per thread, the loads of both first.
-        // chunk c: row ((c >> 6) << 3) | (c & 7), K offset ((c >> 3) & 7) * 8, so
-        // eight lanes write one 128-byte core-matrix row group (no bank conflict)
-        {
-          static_assert(128 * (kRf2KC / 8) == 2 * kDelNT, "two H' chunks per thread");
-          float x[2][8];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int c = tid + u * kDelNT;
-            const int i = rb * 128 + (((c >> 6) << 3) | (c & 7)), k0 = kc * kRf2KC + (((c >> 3) & 7) << 3);
-            rf_ld8(G + (size_t)(i < L ? i : 0) * L + k0, i < L ? L - k0 : 0, vec, x[u]);
-          }
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int c = tid + u * kDelNT;
-            const int r = ((c >> 6) << 3) | (c & 7), m0 = ((c >> 3) & 7) << 3;
-            const int i = rb * 128 + r;
-            const float cp = (i < L && sig * s[i] > 0) ? cpl0 : cpl1;
-            uint32_t h[4], l[4];
-#pragma unroll
-            for (int t = 0; t < 8; t += 2) {
-              const float xa = rintf(x[u][t] * cp * sH) * 0x1p-14f, xb = rintf(x[u][t + 1] * cp * sH) * 0x1p-14f;
-              h[t / 2] = f32x2_to_f16x2(xa, xb);
-              l[t / 2] = f32x2_to_f16x2(xa - f16_lo_to_f32(h[t / 2]), xb - f16_hi_to_f32(h[t / 2]));
-            }
-            const uint32_t off = rf_off2(r, m0);
-            *reinterpret_cast<uint4*>(sa + off) = make_uint4(h[0], h[1], h[2], h[3]);
-            *reinterpret_cast<uint4*>(sa + 128 * kRf2KC * 2 + off) = make_uint4(l[0], l[1], l[2], l[3]);
-          }
-        }
-        }
-        // B: E^T (row n = column n of E, K = rows of E) x 2^se, hi / lo;
-        // wsE holds E^T, so a chunk is eight consecutive words of row n (two
-        // float4 loads: ldE and the offsets are multiples of four); two
-        // chunks per thread in flight
-        const int nc2 = Lp * (kRf2KC / 8);
-        for (int c0 = tid; c0 < nc2; c0 += 2 * kDelNT) {
-          float x[2][8];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int c = c0 + u * kDelNT;
-            const int n = ((c >> 6) << 3) | (c & 7), k0 = kc * kRf2KC + (((c >> 3) & 7) << 3);
-            const bool ok = c < nc2 && n < L;
-            rf_ld8(wsE + (size_t)(ok ? n : 0) * ldE + k0, ok ? ldE - k0 : 0, true, x[u]);
-          }
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int c = c0 + u * kDelNT;
-            if (c < nc2) {
-              const int n = ((c >> 6) << 3) | (c & 7), m0 = ((c >> 3) & 7) << 3;
-              uint32_t h[4], l[4];
-#pragma unroll
-              for (int t = 0; t < 8; t += 2) {
-                const float xa = x[u][t] * sE, xb = x[u][t + 1] * sE;
-                h[t / 2] = f32x2_to_f16x2(xa, xb);
-                l[t / 2] = f32x2_to_f16x2(xa - f16_lo_to_f32(h[t / 2]), xb - f16_hi_to_f32(h[t / 2]));
-              }
-              const uint32_t off = rf_off2(n, m0);
-              unsigned char* bp = sm + nr * kAbuf;
-              *reinterpret_cast<uint4*>(bp + off) = make_uint4(h[0], h[1], h[2], h[3]);
-              *reinterpret_cast<uint4*>(bp + bl + off) = make_uint4(l[0], l[1], l[2], l[3]);
-            }
-          }
-        }
-        fence_async_smem();
-        tc_fence_before();
-        __syncthreads();
-        if (tid == 0) {
-          tc_fence_after();
-#pragma unroll 1
-          for (int ur = 0; ur < nr; ++ur)
-#pragma unroll 1
-          for (int half = 0; half * 256 < Lp; ++half) {
-            const int Nh = Lp - half * 256 < 256 ? Lp - half * 256 : 256;
-            const uint32_t idesc2 = make_idesc_f16(Nh);
-            const uint32_t bo = (uint32_t)half * 32u * 1024u;  // 256 rows of B: 32 groups of 8 x 1024 B
-            const uint32_t a2 = sm0 + (uint32_t)ur * kAbuf;
-#pragma unroll 1
-            for (int kk = 0; kk < kRf2KC / 16; ++kk) {
-              const uint32_t ko = (uint32_t)kk * 256u;
-              const uint32_t d = tc->tmem + (uint32_t)((ur + half) * 256);
-              const uint64_t ahi = make_smem_desc(a2 + ko, 128u, (kRf2KC / 8) * 128u);
-              const uint64_t bhi = make_smem_desc(b2 + bo + ko, 128u, (kRf2KC / 8) * 128u);
-              tc_mma_f16(d, ahi, bhi, idesc2, (kc > 0 || kk > 0) ? 1 : 0);
-              tc_mma_f16(d, ahi, bhi + (uint64_t)(bl >> 4), idesc2, 1);
-              tc_mma_f16(d, ahi + (uint64_t)((128u * kRf2KC * 2u) >> 4), bhi, idesc2, 1);
-            }
-          }
-        }
-        if (!tc_commit_wait(tc)) {
-          if (tid == 0) atomicOr(status, kStatusTimeout);
-          tc->failed = 1;
-          tc->cphase = ph;
-          return -1.f;
-        }
-      }
-      // epilogue: rows rb*128 + 32 q4 + lane of each row block of the group
-      // (its accumulator at TMEM column 256 ur); columns in groups of eight
-      // (one TMEM load each), two groups 32 apart per pass, loads first
-#pragma unroll 1
-      for (int ur = 0; ur < nr; ++ur) {
-      const int rb = rb0 + ur;
-      const int i = rb * 128 + 32 * q4 + lane;
-      const bool up = i < L && sig * s[i] > 0;
-      const float cp = up ? cpl0 : cpl1, cmh = up ? cmh0 : cmh1, cml = up ? cml0 : cml1;
-      float* Gi = G + (size_t)(i < L ? i : 0) * L;
-#pragma unroll 1
-      for (int col0 = 8 * g4; col0 < Lp; col0 += 64) {
-        float q[2][8], go[2][8];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) rf_ld8(Gi + col0 + 32 * u, i < L ? L - col0 - 32 * u : 0, vec, go[u]);
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          if (col0 + 32 * u < Lp) {  // warp-uniform
-            tmem_ld8(tc->tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(256 * ur + col0 + 32 * u), q[u]);
-          } else {
-#pragma unroll
-            for (int c = 0; c < 8; ++c) q[u][c] = 0.f;
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int nv = i < L ? L - col0 - 32 * u : 0;
-#pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            const float Hp = rintf(go[u][c] * cp * sH) * sHi;
-            const float y = Hp + q[u][c] * sQ;
-            q[u][c] = fmaf(y, cmh, y * cml);
-            if (c < nv) drift = fmaxf(drift, fabsf(go[u][c] - q[u][c]));
-          }
-          rf_st8(Gi + col0 + 32 * u, nv, vec, q[u]);
-        }
-      }
-      }
-      tc_fence_before();
-      __syncthreads();
-    }
-    *steps += 1;
-    if (emax <= 0x1p-13f) break;
+    drift = fmaxf(drift, rf_update(P, sm, eh, se, W));
+    if (W.bad || emax <= 0x1p-13f) break;
+    fence_async_smem();
+    __syncthreads();
   }
-  tc->cphase = ph;
-  return rf_block_max(drift, red);
+  __syncthreads();
+  if (threadIdx.x == 0) *sync = P.sync;
+  if (W.bad) {  // uniform: every thread has left together
+    if (threadIdx.x == 0) atomicOr(status, kStatusTimeout);
+    tc->failed = 1;
+    return -1.f;
+  }
+  const float d = rf_block_max(drift, red);
+  return ok ? d : -1.f;
 }
 
-// G_dn = 1 - G_up^T for a particle-hole symmetric bath (both L x L FP32 in
-// global memory), through per-warp 32 x 33 shared-memory tiles (tile: 16
+// G_dn = 1 - G_up^T for a particle-hole symmetric bath (both L x L FP32 at row
+// stride ld), through per-warp 32 x 33 shared-memory tiles (tile: 16
 // warps x 32 x 33 floats) so that reads and writes are both coalesced.  The
 // rows of a tile go in batches of 16 with every load of a batch (G_up, and
 // the old G_dn for the drift) issued before its stores.
 // Returns max |G_dn(old) - G_dn(new)| (block-wide).  All threads call it.
-__device__ inline float ph_mirror(const float* Gu, float* Gd, int L, float* tile, float* red) {
+__device__ inline float ph_mirror(const float* Gu, float* Gd, int L, int ld, float* tile, float* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int NW = kDelNT / 32;
   float* tw = tile + warp * 32 * 33;
@@ -571,7 +888,7 @@ __device__ inline float ph_mirror(const float* Gu, float* Gd, int L, float* tile
 #pragma unroll
       for (int r = 0; r < 16; ++r) {
         const int i = ti * 32 + h + r;
-        v[r] = (i < L && c < L) ? Gu[(size_t)i * L + c] : 0.f;
+        v[r] = (i < L && c < L) ? Gu[(size_t)i * ld + c] : 0.f;
       }
 #pragma unroll
       for (int r = 0; r < 16; ++r) tw[(h + r) * 33 + lane] = v[r];
@@ -583,7 +900,7 @@ __device__ inline float ph_mirror(const float* Gu, float* Gd, int L, float* tile
 #pragma unroll
       for (int r = 0; r < 16; ++r) {
         const int i = tj * 32 + h + r;  // destination row = source column
-        o[r] = (i < L && cc < L) ? Gd[(size_t)i * L + cc] : 0.f;
+        o[r] = (i < L && cc < L) ? Gd[(size_t)i * ld + cc] : 0.f;
       }
 #pragma unroll
       for (int r = 0; r < 16; ++r) {
@@ -591,7 +908,7 @@ __device__ inline float ph_mirror(const float* Gu, float* Gd, int L, float* tile
         if (i < L && cc < L) {
           const float gn = (i == cc ? 1.f : 0.f) - tw[lane * 33 + h + r];
           drift = fmaxf(drift, fabsf(o[r] - gn));
-          Gd[(size_t)i * L + cc] = gn;
+          Gd[(size_t)i * ld + cc] = gn;
         }
       }
     }

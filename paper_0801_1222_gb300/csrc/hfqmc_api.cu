@@ -37,7 +37,7 @@ struct GridHost {
   int k_req = 0;        // the delay depth asked for (option or table), before fitting
   int k1 = 0, ub1 = 2;  // k and U blocks of the G_up-only sweep's layout (one spin's panels)
   bool refine = false;  // recompute by Newton refinement (FP32 delayed path)
-  uint16_t* d_aslc = nullptr;  // its slice table of A (device)
+  uint16_t* d_tab = nullptr;   // its slice table of A (device)
   bool g0_set = false, ever_set = false;
   long long out_off;
 };
@@ -465,7 +465,7 @@ int create_impl(hfqmc_ctx** out, double beta, const double* U, bool per_grid_U,
     off += align256(bytes);
     return o2;
   };
-  std::vector<size_t> offM(n_grids), offG0(n_grids), offMinv(n_grids), offRc(n_grids), offAsl(n_grids);
+  std::vector<size_t> offM(n_grids), offG0(n_grids), offMinv(n_grids), offRc(n_grids), offTab(n_grids);
   for (int g = 0; g < n_grids; ++g) {
     offM[g] = take(sizeof(double) * (size_t)c->gh[g].L * c->gh[g].L);
     offG0[g] = take(sizeof(double) * (size_t)c->gh[g].L);
@@ -474,7 +474,7 @@ int create_impl(hfqmc_ctx** out, double beta, const double* U, bool per_grid_U,
   for (int g = 0; g < n_grids; ++g)
     if (c->gh[g].refine) {
       offRc[g] = take(sizeof(RefineConst));
-      offAsl[g] = take(rf_aslc_bytes(c->gh[g].L));
+      offTab[g] = take(rf_tab_bytes(c->gh[g].L));
     }
   struct ItemOff {
     size_t s, G, ws, acc, bins, accD, cnt;
@@ -539,16 +539,12 @@ int create_impl(hfqmc_ctx** out, double beta, const double* U, bool per_grid_U,
     c->gc[g].rc = nullptr;
     if (c->gh[g].refine) {
       // the field-independent parts; ea and the slices come with each bath (set_G0)
-      const int L = c->gh[g].L;
       const double lam = c->gh[g].lambda;
       RefineConst r;
       std::memset(&r, 0, sizeof(r));
-      c->gh[g].d_aslc = (uint16_t*)(c->d_pool + offAsl[g]);
-      r.aslc = c->gh[g].d_aslc;
-      r.nrb = (L + 127) / 128;
-      r.nkc = (L + kRfKC - 1) / kRfKC;
+      c->gh[g].d_tab = (uint16_t*)(c->d_pool + offTab[g]);
+      r.tab = c->gh[g].d_tab;
       r.emax_step = o.refine_max == 0.0 ? 0.00390625f : (o.refine_max < 0.0 ? -1.f : (float)o.refine_max);
-      r.nN = (L + 79) / 80 * 80 < (L + 63) / 64 * 64 ? 80 : 64;
       r.cplus[0] = (float)std::exp(lam);
       r.cplus[1] = (float)std::exp(-lam);
       for (int v = 0; v < 2; ++v) {
@@ -769,7 +765,7 @@ int hfqmc_set_G0(hfqmc_ctx* c, int grid, const double* G0_tau) {
   if (c->gc[grid].rc) {
     // the refinement's slices of A = M^{-1} - diag(...) for this bath
     RefineConst* rc = const_cast<RefineConst*>(c->gc[grid].rc);
-    r = launch_refine_prep(h.L, c->gc[grid].Minv, h.lambda, rc, h.d_aslc, c->stream);
+    r = launch_refine_prep(h.L, c->gc[grid].Minv, h.lambda, rc, h.d_tab, c->stream);
     if (r) return cuda_fail(c, (cudaError_t)r, "refinement slice kernel");
   }
   SweepArgs a;

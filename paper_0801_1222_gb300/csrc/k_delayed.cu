@@ -36,6 +36,58 @@ constexpr int kRowsPerThread = 2;  // rows t/2 + 256 q, q < 2: L <= 512
 constexpr int kRowStride = kDelNT / 2;
 constexpr int kNoSlice = 0x7fffffff;
 
+// Where a chain stands between two stretches of its sweeps (see the kernel)
+struct SweepPos {
+  long long n_acc;
+  unsigned long long hash;  // kept up to date by one thread, for the chain's decision hash
+  long long t0;             // global index of the call's first sweep
+  uint32_t sw;
+  int l, par;
+  float fu, fd;
+};
+// What its recomputes have added up to
+struct RecTotals {
+  double drift;
+  long long n_rec;
+  int n_fb;  // handed to Gauss-Jordan by the refinement
+};
+
+// A chain's constants, in shared memory, and what follows from them.  Each
+// scope of the kernel takes its own copy, so that only what it uses is in
+// registers there.
+struct ChainConst {
+  GridConst gc;
+  ItemPtrs ip;
+  DelLayout lay;
+};
+constexpr int kChainOff = kRowsPerThread * kRowStride;  // the field takes L <= 512 bytes
+static_assert(kChainOff + sizeof(ChainConst) <= 1024, "the head ends at off_body = 1024");
+struct ChainView {
+  GridConst gc;
+  ItemPtrs ip;
+  DelLayout lay;
+  int L, ld;
+  bool resident;
+  float *Ggl, *Gu, *Gd;  // G in HBM; the G the sweep works on (row pitch ld)
+  int8_t* ss;            // the field, in shared memory
+  __device__ __forceinline__ ChainView(const ChainConst& c, unsigned char* smem) : gc(c.gc), ip(c.ip), lay(c.lay) {
+    L = gc.L;
+    resident = gc.resident != 0;
+    ld = resident ? lay.ldS : L;
+    Ggl = reinterpret_cast<float*>(ip.G);
+    Gu = resident ? reinterpret_cast<float*>(smem + lay.off_G) : Ggl;
+    Gd = Gu + (size_t)L * ld;
+    ss = reinterpret_cast<int8_t*>(smem + lay.off_s);
+  }
+};
+
+// A chain runs as stretches of sweeping between recomputes.  Everything a
+// stretch needs is re-derived at its start -- the field from shared memory,
+// the uniforms from Philox, the diagonal from G, the rest from SweepPos -- so
+// that no sweep state is live across the recompute: its code, which needs
+// every register itself, leaves the accept loop's registers alone (with the
+// refinement inside the loop the compiler spilled 300 bytes of both).
+//
 // kRecord: every accepted flip also sets its bit in the chain's decision
 // trace (a.trace_mode == kTraceRecord), for replay by an FP64 run.
 // kRefine: the recompute tries the Newton refinement (grids with a
@@ -60,12 +112,19 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
   __shared__ int s_next[3];  // next accepted slice, triple-buffered (see take_next)
   __shared__ int s_bad;
   __shared__ uint32_t s_tmem_base;
-  __shared__ __align__(8) unsigned long long s_mbar[5];
+  __shared__ __align__(8) unsigned long long s_mbar[12];
+  __shared__ RfSync s_rf;
+  __shared__ SweepPos s_pos;
+  __shared__ RecTotals s_rec;
+  // in the head of dynamic shared memory, behind the field (static shared memory is kept to
+  // the 512 bytes that kSmemCap leaves)
+  ChainConst& s_chain = *reinterpret_cast<ChainConst*>(smem + kChainOff);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool use_tc = a.flush != 2;
   TcState tc;
   if (use_tc) tc_setup(&tc, &s_tmem_base, s_mbar, a.status);
+  if (tid == 0) s_rf = RfSync{0u, 0u, 0u};
 
   for (;;) {
     if (tid == 0) s_item = atomicAdd(a.queue_head, 1);
@@ -73,34 +132,54 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
     const int q = s_item;
     __syncthreads();
     if (q >= a.n_items) break;
-    const ItemPtrs ip = a.items[a.order[q]];
-    const GridConst gc = a.grids[ip.grid];
-    const int L = gc.L, K = gc.k;
-    const bool resident = gc.resident != 0;
-    const DelLayout lay =
-        del_layout(L, K, resident, gc.gj_smem != 0, gc.gtile != 0, gc.ub, gc.rc != nullptr, kMirror ? 1 : 2);
+    if (tid == 0) {
+      s_chain.ip = a.items[a.order[q]];
+      s_chain.gc = a.grids[s_chain.ip.grid];
+      const GridConst& gc = s_chain.gc;
+      s_chain.lay = del_layout(gc.L, gc.k, gc.resident != 0, gc.gj_smem != 0, gc.gtile != 0, gc.ub, gc.rc != nullptr,
+                               kMirror ? 1 : 2);
+    }
+    __syncthreads();
+    {
+    const ChainView v(s_chain, smem);
+    const GridConst& gc = v.gc;
+    const ItemPtrs& ip = v.ip;
+    const DelLayout& lay = v.lay;
+    const int L = v.L, ld = v.ld;
+    const bool resident = v.resident;
+    float *const Ggl = v.Ggl, *const Gu = v.Gu, *const Gd = v.Gd;
+    int8_t* const ss = v.ss;
+    if (resident) {
+      for (int i = warp; i < (kMirror ? 1 : 2) * L; i += NW)
+        for (int jj = lane; jj < L; jj += 32) Gu[(size_t)i * ld + jj] = Ggl[(size_t)i * L + jj];
+    }
+    for (int l = tid; l < L; l += NT) ss[l] = ip.s[l];
+    if (tid < 3) s_next[tid] = kNoSlice;
+    if (tid == 0) {
+      s_bad = 0;
+      s_pos = SweepPos{ip.cnt->accepted, ip.cnt->hash, ip.cnt->t, 0u, -1, 0, 0.f, 0.f};
+      s_rec = RecTotals{ip.cnt->drift, 0, 0};
+    }
+    __syncthreads();
+    }
+
+    for (;;) {
+    bool done, recompute;
+    {  // a stretch of sweeping
+    const ChainView v(s_chain, smem);
+    const GridConst& gc = v.gc;
+    const ItemPtrs& ip = v.ip;
+    const DelLayout& lay = v.lay;
+    const int L = v.L, ld = v.ld;
+    const bool resident = v.resident;
+    float *const Ggl = v.Ggl, *const Gu = v.Gu, *const Gd = v.Gd;
+    int8_t* const ss = v.ss;
+    const int K = gc.k;
     // product tile buffer of the TMA reduce flush (G in HBM, tensor map set)
     float* dtile = gc.gtile ? reinterpret_cast<float*>(smem + lay.off_gtile) : nullptr;
-
-    float* Ggl = reinterpret_cast<float*>(ip.G);
-    float* Gu;
-    float* Gd;
-    int ld;
-    if (resident) {
-      ld = lay.ldS;
-      Gu = reinterpret_cast<float*>(smem + lay.off_G);
-      Gd = Gu + (size_t)L * ld;
-    } else {
-      ld = L;
-      Gu = Ggl;
-      Gd = Ggl + (size_t)L * L;
-    }
     float* Pu = reinterpret_cast<float*>(smem + lay.off_U);  // [2][L][KP] (spin stride padded): U panels
     float* Pw = reinterpret_cast<float*>(smem + lay.off_W);  // [2][L][KP]: W panels
     float* fac = reinterpret_cast<float*>(smem + lay.off_diag);  // [L][2]: flip factors of candidates
-    double* colk = reinterpret_cast<double*>(smem + lay.off_colk);
-    int* perm = reinterpret_cast<int*>(smem + lay.off_perm);
-    int8_t* ss = reinterpret_cast<int8_t*>(smem + lay.off_s);
     unsigned char* stage = smem + lay.off_stage;
     const int KP = lay.KP;
     const int panel_floats4 = del_panel_floats(L, KP, kMirror ? 1 : 2) / 4;  // one panel, the kept spins
@@ -111,16 +190,7 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
     };
     const float d0 = gc.deltaf[0], d1 = gc.deltaf[1];
     const int rule = a.accept_rule;
-
-    if (resident) {
-      for (int i = warp; i < 2 * L; i += NW)
-        for (int jj = lane; jj < L; jj += 32) Gu[(size_t)i * ld + jj] = Ggl[(size_t)i * L + jj];
-    }
-    for (int l = tid; l < L; l += NT) ss[l] = ip.s[l];
-    if (tid < 3) s_next[tid] = kNoSlice;
-    if (tid == 0) s_bad = 0;
-    __syncthreads();
-
+    const uint32_t n_sweeps = (uint32_t)(a.n_warm + a.n_meas), n_warm = (uint32_t)a.n_warm;  // at most 2^31 a call
     // per-thread row state: this spin's current diagonal, field, this sweep's uniform
     const int sp = tid & 1;
     const int row0 = tid >> 1;
@@ -142,6 +212,18 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
         if (r < L) dg[qq] = Gs[(size_t)r * ld + r];
       }
     };
+    uint32_t sw = s_pos.sw;
+    int l = s_pos.l;  // next accepted slice; -1: the sweep begins
+    int par = s_pos.par;  // s_next buffer of the current round
+    float fu = s_pos.fu, fd = s_pos.fd;  // its flip factors
+    auto draw_uniforms = [&](long long t) {
+#pragma unroll
+      for (int qq = 0; qq < kRowsPerThread; ++qq) {
+        if (qq * kRowStride >= L) break;  // uniform: rows beyond the grid
+        const int r = row0 + qq * kRowStride;
+        if (r < L) uv[qq] = proposal_uniform_f32(r, t, ip.chain, ip.grid, a.seed);
+      }
+    };
 #pragma unroll
     for (int qq = 0; qq < kRowsPerThread; ++qq) {
       if (qq * kRowStride >= L) break;  // uniform: rows beyond the grid
@@ -151,22 +233,17 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
       lastbad[qq] = false;
       dg[qq] = 0.f;
     }
+    if (l >= 0) draw_uniforms(s_pos.t0 + sw);  // mid-sweep: this sweep's uniforms again
     load_diag();
-    zero_panels();
-
-    const ChainCounters c0 = *ip.cnt;
-    long long n_acc = c0.accepted;
+    zero_panels();  // also after a recompute, whose workspace may have overlaid them
     // accepted flips until the next recompute (the cumulative count reaches a
-    // multiple of n_wrap); counted down so the hot loop needs no 64-bit modulo
-    int until_rec = gc.n_wrap > 0 ? (int)(gc.n_wrap - n_acc % gc.n_wrap) : 0;
-    long long n_rec = 0, n_bad = 0;
-    int n_fb = 0;  // recomputes the refinement handed to Gauss-Jordan
-    unsigned long long hash = c0.hash;
-    double drift = c0.drift;
-    const long long n_sweeps = a.n_warm + a.n_meas;
+    // multiple of n_wrap), or the longest stretch when there is none; counted
+    // down so the hot loop needs no 64-bit count
+    const int stretch = gc.n_wrap > 0 ? (int)(gc.n_wrap - s_pos.n_acc % gc.n_wrap) : 0x7fffffff;
+    int left = stretch;
+    int n_bad = 0;
     int j = 0;     // pending flips in the panels
     uint32_t exq = 0u;  // biased exponents of this thread's largest appended |u| (byte 0), |w| (byte 1)
-    int par = 0;   // s_next buffer of the current round
     __syncthreads();
 
     // G += U W^T for both spins, then the diagonals are re-read from G.
@@ -242,23 +319,18 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
       return nxt;
     };
 
-    for (long long sw = 0; sw < n_sweeps; ++sw) {
-      const long long t = c0.t + sw;
-#pragma unroll
-      for (int qq = 0; qq < kRowsPerThread; ++qq) {
-        if (qq * kRowStride >= L) break;  // uniform: rows beyond the grid
-        const int r = row0 + qq * kRowStride;
-        if (r < L) uv[qq] = proposal_uniform_f32(r, t, ip.chain, ip.grid, a.seed);
-      }
-      propose(0);
-      __syncthreads();
-      int l = take_next(0);
-      // flip factors of the accepted slice; read before any flush or
-      // recompute, whose shared-memory workspace may overlay fac[]
-      float fu = 0.f, fd = 0.f;
-      if (l < L) {
-        fu = fac[2 * l];
-        fd = fac[2 * l + 1];
+    for (; sw < n_sweeps; ++sw) {
+      if (l < 0) {
+        draw_uniforms(s_pos.t0 + sw);
+        propose(0);
+        __syncthreads();
+        l = take_next(0);
+        // flip factors of the accepted slice; read before any flush or
+        // recompute, whose shared-memory workspace may overlay fac[]
+        if (l < L) {
+          fu = fac[2 * l];
+          fd = fac[2 * l + 1];
+        }
       }
       while (l < L) {
         if constexpr (kMirror) {
@@ -361,11 +433,12 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
           }
         }
         }
-        hash = (hash ^ (unsigned long long)(t * (long long)L + l)) * kFnvPrime;
+        // the decision hash by the last thread (which owns no row for L <= 255)
+        if (tid == NT - 1)
+          s_pos.hash = (s_pos.hash ^ (unsigned long long)((s_pos.t0 + sw) * (long long)L + l)) * kFnvPrime;
         if constexpr (kRecord) {
           if (tid == 0) ip.trace[(size_t)sw * trace_words(L) + (l >> 5)] |= 1u << (l & 31);
         }
-        ++n_acc;
         ++j;
         propose(l + 1);
         __syncthreads();
@@ -376,63 +449,18 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
           fd_next = fac[2 * lnext + 1];
         }
         if (j == K) flush();
-        if (gc.n_wrap > 0 && --until_rec == 0) {
-          until_rec = gc.n_wrap;
-          flush();
-          double d = -1.0;
-          // G in HBM while the refinement runs (its staging overlays the whole
-          // body of shared memory, a resident G included)
-          bool in_hbm = false;
-          if (kRefine && gc.rc && use_tc && !tc.failed && gc.lambda != 0.0) {
-            if (resident) {
-              for (int i = warp; i < 2 * L; i += NW)
-                for (int jj = lane; jj < L; jj += 32) Ggl[(size_t)i * L + jj] = Gu[(size_t)i * ld + jj];
-              __syncthreads();
-              in_hbm = true;
-            }
-            int steps = 0;
-            float* rws = reinterpret_cast<float*>(ip.ws);
-            float* rred = reinterpret_cast<float*>(red);
-            const float d0 = refine_spin(gc, *gc.rc, ss, 1, Ggl, rws, smem + lay.off_rf, &tc, rred, a.status, &steps);
-            // spin down: not kept during a mirrored sweep; mirrored for a
-            // particle-hole symmetric bath, else refined too
-            const float d1 = d0 < 0.f ? -1.f
-                             : kMirror ? 0.f
-                             : gc.ph   ? ph_mirror(Ggl, Ggl + (size_t)L * L, L,
-                                                   reinterpret_cast<float*>(smem + lay.off_rf), rred)
-                                       : refine_spin(gc, *gc.rc, ss, -1, Ggl + (size_t)L * L, rws, smem + lay.off_rf,
-                                                     &tc, rred, a.status, &steps);
-            if (d0 >= 0.f && d1 >= 0.f)
-              d = fmax((double)d0, (double)d1);
-            else
-              ++n_fb;
-          }
-          if (d < 0.0) {
-            // from scratch: FP64 workspace in HBM, inverted by panels whose
-            // scratch overlays the idle part of shared memory (never G)
-            d = recompute_green_inv<float, NT, true>(
-                gc, ss, in_hbm ? Ggl : Gu, in_hbm ? Ggl + (size_t)L * L : Gd, in_hbm ? L : ld, ip.ws, red, redi,
-                &s_inv, &s_piv, colk, perm, true, a.status, 0, kMirror ? 1 : 2,
-                reinterpret_cast<double*>(smem + lay.off_gjb));
-          }
-          if (in_hbm) {
-            for (int i = warp; i < 2 * L; i += NW)
-              for (int jj = lane; jj < L; jj += 32) Gu[(size_t)i * ld + jj] = Ggl[(size_t)i * L + jj];
-            __syncthreads();
-          }
-          drift = fmax(drift, d);
-          ++n_rec;
-          zero_panels();  // the recompute's workspace may have overlaid them
-          load_diag();
-          __syncthreads();
-        }
         l = lnext;
         fu = fu_next;
         fd = fd_next;
+        if (--left == 0) break;
       }
-      if (sw >= a.n_warm) {
+      if (left == 0) {
         flush();
-        const long long m = sw - a.n_warm;
+        break;
+      }
+      if (sw >= n_warm) {
+        flush();
+        const long long m = sw - n_warm;
         const int b = (int)((kBins * m) / a.n_meas);
         // partial sums in the (idle) staging area, totals in the panels' space
         float* part = reinterpret_cast<float*>(smem + lay.off_stage);
@@ -471,38 +499,125 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
           ip.accD[1 + b] = d1 + (double)v / (double)L;
         }
       }
+      l = -1;
       __syncthreads();
     }
+    // bad ratios were counted per owned row: sum over the CTA
+    {
+      const int nb = __reduce_add_sync(0xffffffffu, n_bad);
+      if (lane == 0 && nb) atomicAdd(&s_bad, nb);
+    }
     flush();
+    if (tid == 0) {
+      s_pos.n_acc += stretch - left;
+      s_pos.sw = sw;
+      s_pos.l = l;
+      s_pos.par = par;
+      s_pos.fu = fu;
+      s_pos.fd = fd;
+    }
+    done = left != 0;
+    recompute = left == 0 && gc.n_wrap > 0;
+    }
+    __syncthreads();
+    if (done) break;
+    if (!recompute) continue;
 
+    {  // a recompute
+    const ChainView v(s_chain, smem);
+    const GridConst& gc = v.gc;
+    const ItemPtrs& ip = v.ip;
+    const DelLayout& lay = v.lay;
+    const int L = v.L, ld = v.ld;
+    const bool resident = v.resident;
+    float *const Ggl = v.Ggl, *const Gu = v.Gu, *const Gd = v.Gd;
+    int8_t* const ss = v.ss;
+    double* colk = reinterpret_cast<double*>(smem + lay.off_colk);
+    int* perm = reinterpret_cast<int*>(smem + lay.off_perm);
+    double d = -1.0;
+    // G in HBM while the refinement runs, where its staging overlays a
+    // resident G (else it works on G where it lies)
+    constexpr int kSpins = kMirror ? 1 : 2;
+    bool in_hbm = false;
+    if (kRefine && gc.rc && use_tc && !tc.failed && gc.lambda != 0.0) {
+      if (resident && !lay.rf_keeps_G) {
+        for (int i = warp; i < kSpins * L; i += NW)
+          for (int jj = lane; jj < L; jj += 32) Ggl[(size_t)i * L + jj] = Gu[(size_t)i * ld + jj];
+        __syncthreads();
+        in_hbm = true;
+      }
+      float* rws = reinterpret_cast<float*>(ip.ws);
+      float* rred = reinterpret_cast<float*>(red);
+      float* Ru = in_hbm ? Ggl : Gu;
+      float* Rd = in_hbm ? Ggl + (size_t)L * L : Gd;
+      const int rld = in_hbm ? L : ld;
+      // spin down: not kept during a mirrored sweep; mirrored for a
+      // particle-hole symmetric bath, else refined too
+      const int n_ref = kMirror || gc.ph ? 1 : 2;
+      float dmax = 0.f;
+#pragma unroll 1
+      for (int r = 0; r < n_ref && dmax >= 0.f; ++r) {
+        const float dr = refine_spin(gc, gc.rc, ss, r ? -1 : 1, r ? Rd : Ru, rld, rws, smem + lay.off_rf, &tc, &s_rf,
+                                     rred, a.status);
+        dmax = dr < 0.f ? -1.f : fmaxf(dmax, dr);
+      }
+      if (!kMirror && gc.ph && dmax >= 0.f)
+        dmax = fmaxf(dmax, ph_mirror(Ru, Rd, L, rld, reinterpret_cast<float*>(smem + lay.off_rf), rred));
+      if (dmax >= 0.f)
+        d = (double)dmax;
+      else if (tid == 0)
+        ++s_rec.n_fb;
+    }
+    if (d < 0.0) {
+      // from scratch: FP64 workspace in HBM, inverted by panels whose
+      // scratch overlays the idle part of shared memory (never G)
+      d = recompute_green_inv<float, NT, true>(
+          gc, ss, in_hbm ? Ggl : Gu, in_hbm ? Ggl + (size_t)L * L : Gd, in_hbm ? L : ld, ip.ws, red, redi,
+          &s_inv, &s_piv, colk, perm, true, a.status, 0, kMirror ? 1 : 2,
+          reinterpret_cast<double*>(smem + lay.off_gjb));
+    }
+    if (in_hbm) {
+      for (int i = warp; i < kSpins * L; i += NW)
+        for (int jj = lane; jj < L; jj += 32) Gu[(size_t)i * ld + jj] = Ggl[(size_t)i * L + jj];
+      __syncthreads();
+    }
+    if (tid == 0) {
+      s_rec.drift = fmax(s_rec.drift, d);
+      ++s_rec.n_rec;
+    }
+    }
+    __syncthreads();
+    }
+
+    const ChainView v(s_chain, smem);
+    const GridConst& gc = v.gc;
+    const ItemPtrs& ip = v.ip;
+    const DelLayout& lay = v.lay;
+    const int L = v.L, ld = v.ld;
+    const bool resident = v.resident;
+    float *const Ggl = v.Ggl, *const Gu = v.Gu, *const Gd = v.Gd;
+    int8_t* const ss = v.ss;
     if (resident) {
-      for (int i = warp; i < 2 * L; i += NW)
+      for (int i = warp; i < (kMirror ? 1 : 2) * L; i += NW)
         for (int jj = lane; jj < L; jj += 32) Ggl[(size_t)i * L + jj] = Gu[(size_t)i * ld + jj];
     }
     if constexpr (kMirror) {
       // the chain's G_dn for the host and the next call: 1 - G_up^T
       __syncthreads();
-      (void)ph_mirror(Ggl, Ggl + (size_t)L * L, L, reinterpret_cast<float*>(smem + lay.off_rf),
+      (void)ph_mirror(Ggl, Ggl + (size_t)L * L, L, L, reinterpret_cast<float*>(smem + lay.off_rf),
                       reinterpret_cast<float*>(red));
     }
     for (int l = tid; l < L; l += NT) ip.s[l] = ss[l];
-    // bad ratios were counted per owned row: sum over the CTA
-    {
-      const int nb = __reduce_add_sync(0xffffffffu, (int)n_bad);
-      if (lane == 0 && nb) atomicAdd(&s_bad, nb);
-      __syncthreads();
-      n_bad = s_bad;
-    }
     if (tid == 0) {
-      ChainCounters c = c0;
-      c.t = c0.t + n_sweeps;
-      c.proposals = c0.proposals + n_sweeps * (long long)L;
-      c.accepted = n_acc;
-      c.recomputes = c0.recomputes + n_rec;
-      c.hash = hash;
-      c.bad = c0.bad + n_bad;
-      c.drift = drift;
-      c.fallbacks = c0.fallbacks + n_fb;
+      ChainCounters c = *ip.cnt;
+      c.t += a.n_warm + a.n_meas;
+      c.proposals += (a.n_warm + a.n_meas) * (long long)L;
+      c.accepted = s_pos.n_acc;
+      c.recomputes += s_rec.n_rec;
+      c.hash = s_pos.hash;
+      c.bad += s_bad;
+      c.drift = s_rec.drift;
+      c.fallbacks += s_rec.n_fb;
       *ip.cnt = c;
     }
     __syncthreads();

@@ -107,19 +107,14 @@ int launch_bath_inverse(int L, const double* M, double* Minv, int* status, cudaS
 }
 
 // Slices of A = M^{-1} - diag(1 - e^{-sigma lambda s_j}) for the Newton
-// refinement (hfq_refine.cuh): every entry x of M^{-1} (padded with zeros to
-// whole 128-row blocks and 64-column chunks) is written as
+// refinement (hfq_refine.cuh): every entry x of M^{-1} is written as
 //   x = 2^ea sum_{p<6} s_p 2^{-7(p+1)} + (remainder below 2^{ea-43}),
 // s_p = rint of the running remainder times 2^7 (|s_0| <= 128, |s_p| <= 64),
-// each an integer held exactly in FP16, stored in the K-major core-matrix
-// layout the tensor-core operand wants (rows of A = M dimension, columns =
-// K).  A_jj depends on the chain's field: its two values are sliced into
-// rc->dslc and patched in per chain; ea covers both.  One block per (row
-// block, K chunk); every block finds the same ea.
-__device__ __forceinline__ uint32_t rf_core_offset(int r, int m) {
-  return (uint32_t)((r >> 3) * (kRfKC / 8) * 128 + (m >> 3) * 128 + (r & 7) * 16 + (m & 7) * 2);
-}
-
+// each an integer held exactly in FP16.  M^{-1} is skew-circulant, so one
+// 8 x 8 core matrix (rows of A = the MMA's N dimension, columns = K) per
+// block diagonal and slice holds it all; entries beyond the matrix's corner
+// diagonals are zero.  The table's main diagonal is A_jj for sigma s_j = +1;
+// the other value's difference goes into rc->dd; ea covers both.
 __device__ __forceinline__ void rf_slice6(double x, int ea, float* q) {
   double y = ldexp(x, kRfBits - ea);
 #pragma unroll
@@ -131,7 +126,7 @@ __device__ __forceinline__ void rf_slice6(double x, int ea, float* q) {
 }
 
 __global__ void __launch_bounds__(256) k_refine_prep(int L, const double* __restrict__ Minv, double lambda,
-                                                     RefineConst* rc, uint16_t* __restrict__ aslc, int nkc) {
+                                                     RefineConst* rc, uint16_t* __restrict__ tab) {
   __shared__ double red[8];
   const int tid = threadIdx.x;
   const double a0 = Minv[0] - (1.0 - exp(-lambda)), a1 = Minv[0] - (1.0 - exp(lambda));
@@ -142,40 +137,30 @@ __global__ void __launch_bounds__(256) k_refine_prep(int L, const double* __rest
   if (m > 0.0) (void)frexp(m, &ea);  // m < 2^ea
   if (blockIdx.x == 0 && tid == 0) {
     rc->ea = ea;
-    float q[kRfSlicesA];
-    rf_slice6(a0, ea, q);
-    for (int p = 0; p < kRfSlicesA; ++p) rc->dslc[0][p] = __half_as_ushort(__float2half_rn(q[p]));
-    rf_slice6(a1, ea, q);
-    for (int p = 0; p < kRfSlicesA; ++p) rc->dslc[1][p] = __half_as_ushort(__float2half_rn(q[p]));
+    float q0[kRfSlicesA], q1[kRfSlicesA];
+    rf_slice6(a0, ea, q0);
+    rf_slice6(a1, ea, q1);
+    for (int p = 0; p < kRfSlicesA; ++p) rc->dd[p] = q1[p] - q0[p];
   }
-  const int rb = blockIdx.x / nkc, kc = blockIdx.x - rb * nkc;
-  uint16_t* tile = aslc + (size_t)blockIdx.x * kRfSlicesA * (kRfTileA / 2);
-  for (int c = tid; c < 128 * (kRfKC / 8); c += 256) {
-    const int r = c / (kRfKC / 8), m0 = (c - r * (kRfKC / 8)) * 8;
-    const int i = rb * 128 + r;
-    uint32_t w[kRfSlicesA][4];
-#pragma unroll
-    for (int t = 0; t < 8; t += 2) {
-      const int j = kc * kRfKC + m0 + t;
-      float q0[kRfSlicesA], q1[kRfSlicesA];
-      rf_slice6(i < L && j < L ? Minv[(size_t)i * L + j] : 0.0, ea, q0);
-      rf_slice6(i < L && j + 1 < L ? Minv[(size_t)i * L + j + 1] : 0.0, ea, q1);
-#pragma unroll
-      for (int p = 0; p < kRfSlicesA; ++p)
-        w[p][t / 2] = (uint32_t)__half_as_ushort(__float2half_rn(q0[p])) |
-                      ((uint32_t)__half_as_ushort(__float2half_rn(q1[p])) << 16);
-    }
-    const uint32_t off = rf_core_offset(r, m0) / 2;
-#pragma unroll
+  const int ncore = rf_ncore(L), nj = rf_nj(L);
+  for (int e = blockIdx.x * 256 + tid; e < ncore * 64; e += gridDim.x * 256) {
+    const int d = 8 * (e / 64 - (nj - 1)) + ((e >> 3) & 7) - (e & 7);  // i - j
+    double x = 0.0;
+    if (d == 0)
+      x = a0;
+    else if (d > 0 && d < L)
+      x = Minv[(size_t)d * L];
+    else if (d < 0 && d > -L)
+      x = Minv[-d];
+    float q[kRfSlicesA];
+    rf_slice6(x, ea, q);
     for (int p = 0; p < kRfSlicesA; ++p)
-      *reinterpret_cast<uint4*>(tile + (size_t)p * (kRfTileA / 2) + off) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
+      tab[(size_t)p * ncore * 64 + e] = __half_as_ushort(__float2half_rn(q[p]));
   }
 }
 
-int launch_refine_prep(int L, const double* Minv, double lambda, RefineConst* rc, uint16_t* aslc,
-                       cudaStream_t st) {
-  const int nrb = rf_pad(L, 128) / 128, nkc = rf_pad(L, kRfKC) / kRfKC;
-  k_refine_prep<<<nrb * nkc, 256, 0, st>>>(L, Minv, lambda, rc, aslc, nkc);
+int launch_refine_prep(int L, const double* Minv, double lambda, RefineConst* rc, uint16_t* tab, cudaStream_t st) {
+  k_refine_prep<<<(rf_ncore(L) * 64 + 255) / 256, 256, 0, st>>>(L, Minv, lambda, rc, tab);
   return (int)cudaGetLastError();
 }
 
