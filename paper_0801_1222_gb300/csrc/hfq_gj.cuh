@@ -24,119 +24,157 @@
 
 namespace hfq {
 
-// In-place Gauss-Jordan on W = [A | B] (L rows, 2L columns, row-major), in
-// shared or global memory.  colk: L doubles of shared scratch (the pivot
-// column of the current step, so the elimination reads it once per row).
-// The elimination keeps the pivot row in registers and updates two rows per
-// warp iteration, loading 2 x kGjChunk values before any store, so each warp
-// has that many independent loads and DFMAs in flight (the FP64 pipe's
-// latency is long on this part) whether W lives in shared memory or in L2.
-// On return the right half holds A^{-1} B.  Returns -1 on a zero pivot
-// (uniformly in all threads), 0 otherwise.
-// columns per lane and chunk: 8 with 8 warps; 4 with 16 warps, whose register
-// budget is half as large (and twice the warps keep as many loads in flight)
-template <int NT>
-__host__ __device__ constexpr int gj_chunk() { return NT >= 512 ? 4 : 8; }
+// An FP64 warp instruction takes 64 cycles of its scheduler on this part
+// (compares included), so beside the L^2 or so DFMAs of an elimination step
+// the rest of it must not use the FP64 pipe: magnitudes are compared as bit
+// patterns, and no lane multiplies for a column that is not there.  Rows go in
+// batches with all loads before the first store and no condition per element
+// (gj_rows), the columns in as many chunks of 32 as there are.  The elimination
+// by one CTA at L = 100 took 1.09 ms a spin on [A | M] in L2 before (every step
+// over 256 columns, FP64 compares in the pivot search); dealt out over CTAs in
+// shared memory (k_noalloc.cu) it takes 0.39 ms for both.
 
+// The pivot of step k: the row of largest |W_ik|, i >= k (ties: the lowest),
+// and the reciprocal of its entry, in *s_piv (-1: zero or NaN) and *s_inv
+// after the barrier that ends it.
 template <int NT>
-__device__ int gj_eliminate(double* W, int L, double* red, int* redi, double* s_inv, int* s_piv,
-                            double* colk) {
-  constexpr int kGjChunk = gj_chunk<NT>();
+__device__ __forceinline__ void gj_pivot(const double* W, int L, int ld, int k, double* red, int* redi, double* s_inv,
+                                         int* s_piv) {
   constexpr int NW = NT / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int ld = 2 * L;
-  for (int k = 0; k < L; ++k) {
-    double best = -1.0;
-    int bi = L;
-    for (int i = k + tid; i < L; i += NT) {
-      const double v = fabs(W[(size_t)i * ld + k]);
-      if (v > best) {
-        best = v;
-        bi = i;
-      }
+  // magnitudes as unsigned integers (the same order for non-negative doubles);
+  // NaN compares as no magnitude, as it would in FP64
+  unsigned long long best = 0ull;
+  int bi = L;
+  auto offer = [&](unsigned long long v, int i) {
+    if (v > best || (v == best && i < bi)) {
+      best = v;
+      bi = i;
     }
-    for (int o = 16; o; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+  };
+  for (int i = k + tid; i < L; i += NT) {
+    const unsigned long long v = __double_as_longlong(W[(size_t)i * ld + k]) & 0x7fffffffffffffffull;
+    if (v > 0ull && v <= 0x7ff0000000000000ull) offer(v, i);
+  }
+  for (int o = 16; o; o >>= 1) {
+    const unsigned long long ov = __shfl_xor_sync(0xffffffffu, best, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+    offer(ov, oi);
+  }
+  if (lane == 0) {
+    reinterpret_cast<unsigned long long*>(red)[warp] = best;
+    redi[warp] = bi;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    best = lane < NW ? reinterpret_cast<const unsigned long long*>(red)[lane] : 0ull;
+    bi = lane < NW ? redi[lane] : L;
+    for (int o = NW / 2; o; o >>= 1) {
+      const unsigned long long ov = __shfl_xor_sync(0xffffffffu, best, o);
       const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > best || (ov == best && oi < bi)) {
-        best = ov;
-        bi = oi;
-      }
+      offer(ov, oi);
     }
     if (lane == 0) {
-      red[warp] = best;
-      redi[warp] = bi;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      double b = red[0];
-      int p = redi[0];
-      for (int w = 1; w < NW; ++w)
-        if (red[w] > b || (red[w] == b && redi[w] < p)) {
-          b = red[w];
-          p = redi[w];
-        }
-      if (!(b > 0.0) || p >= L) {
+      if (best == 0ull || bi >= L) {
         *s_piv = -1;
       } else {
-        *s_piv = p;
-        *s_inv = 1.0 / W[(size_t)p * ld + k];
+        *s_piv = bi;
+        *s_inv = 1.0 / W[(size_t)bi * ld + k];
       }
     }
-    __syncthreads();
+  }
+  __syncthreads();
+}
+
+// Rows i != k, columns j, j + 32, ... (NC of them; the last one, jl, clamped to
+// the matrix and stored only when it lies in it): W_ij -= colk_i rk_j, R rows a
+// batch with every load before the first store.  zk: column k starts from 0
+// (the identity column folded in).
+template <int NC, int R>
+__device__ __forceinline__ int gj_rows(double* W, int L, int ld, const double* colk, const double (&rk)[NC], int j,
+                                       int jl, bool in, int k, bool zk, int i0, int NW) {
+  for (; i0 + (R - 1) * NW < L; i0 += R * NW) {
+    double v[R][NC], f[R];
+    double* w = W + (size_t)i0 * ld;
+    const size_t step = (size_t)NW * ld;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = i0 + r * NW;
+      f[r] = i != k ? colk[i] : 0.0;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) v[r][c] = w[r * step + (c + 1 < NC ? j + 32 * c : jl)];
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) v[r][c] = fma(-f[r], rk[c], zk && j + 32 * c == k ? 0.0 : v[r][c]);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (i0 + r * NW != k) {
+#pragma unroll
+        for (int c = 0; c + 1 < NC; ++c) w[r * step + j + 32 * c] = v[r][c];
+        if (in) w[r * step + jl] = v[r][NC - 1];
+      }
+  }
+  return i0;
+}
+template <int NT, int NC>
+__device__ __forceinline__ void gj_columns(double* W, int L, int ld, int jend, const double* colk, int c0, int k,
+                                           bool zk) {
+  constexpr int NW = NT / 32, R = NT >= 512 ? 2 : 4;  // 16 warps have half the registers each
+  const int j = c0 + (threadIdx.x & 31), jl = min(j + 32 * (NC - 1), jend - 1);
+  const bool in = j + 32 * (NC - 1) < jend;
+  const double* wk = W + (size_t)k * ld;
+  double rk[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) rk[c] = wk[c + 1 < NC ? j + 32 * c : jl];
+  int i0 = threadIdx.x >> 5;
+  i0 = gj_rows<NC, R>(W, L, ld, colk, rk, j, jl, in, k, zk, i0, NW);
+  gj_rows<NC, 1>(W, L, ld, colk, rk, j, jl, in, k, zk, i0, NW);
+}
+// Columns [j0, jend) of every row but k.
+template <int NT>
+__device__ __forceinline__ void gj_step(double* W, int L, int ld, int j0, int jend, const double* colk, int k, bool zk) {
+#pragma unroll 1
+  for (int c0 = j0; c0 < jend; c0 += 128) {
+    const int n = jend - c0;
+    if (n > 96)
+      gj_columns<NT, 4>(W, L, ld, jend, colk, c0, k, zk);
+    else if (n > 64)
+      gj_columns<NT, 3>(W, L, ld, jend, colk, c0, k, zk);
+    else if (n > 32)
+      gj_columns<NT, 2>(W, L, ld, jend, colk, c0, k, zk);
+    else
+      gj_columns<NT, 1>(W, L, ld, jend, colk, c0, k, zk);
+  }
+}
+
+// In-place Gauss-Jordan on W = [A | B] (L rows, ncol columns of pitch ld, A the
+// first L), in shared or global memory.  colk: L doubles of shared scratch
+// (the pivot column of the current step, so the elimination reads it once per
+// row).  On return the right part holds A^{-1} B.  Returns -1 on a zero pivot
+// (uniformly in all threads), 0 otherwise.
+template <int NT>
+__device__ int gj_eliminate(double* W, int L, int ncol, int ld, double* red, int* redi, double* s_inv, int* s_piv,
+                            double* colk) {
+  const int tid = threadIdx.x;
+  for (int k = 0; k < L; ++k) {
+    gj_pivot<NT>(W, L, ld, k, red, redi, s_inv, s_piv);
     const int p = *s_piv;
     if (p < 0) return -1;
     const double inv = *s_inv;
     // swap rows k and p (columns >= k), scale the new row k; record column k
-    for (int j = k + tid; j < ld; j += NT) {
+    for (int i = tid; i < L; i += NT)
+      if (i != k && i != p) colk[i] = W[(size_t)i * ld + k];
+    for (int j = k + tid; j < ncol; j += NT) {
       const double a = W[(size_t)k * ld + j];
       const double b = W[(size_t)p * ld + j];
       W[(size_t)p * ld + j] = a;
       W[(size_t)k * ld + j] = b * inv;
       if (j == k) colk[p] = a;
     }
-    for (int i = tid; i < L; i += NT)
-      if (i != k && i != p) colk[i] = W[(size_t)i * ld + k];
     __syncthreads();
-    // eliminate column k from every other row
-    const int j0 = k + 1;
-    const double* wk = W + (size_t)k * ld;
-    for (int c0 = j0; c0 < ld; c0 += 32 * kGjChunk) {
-      double rk[kGjChunk];
-#pragma unroll
-      for (int c = 0; c < kGjChunk; ++c) {
-        const int j = c0 + lane + 32 * c;
-        rk[c] = j < ld ? wk[j] : 0.0;
-      }
-      // two rows per warp iteration: 2 x kGjChunk independent DFMAs between
-      // the loads and the stores, enough to cover the FP64 pipe's latency
-      for (int i = warp; i < L; i += 2 * NW) {
-        const int i2 = i + NW;
-        const bool has2 = i2 < L;
-        double v1[kGjChunk], v2[kGjChunk];
-#pragma unroll
-        for (int c = 0; c < kGjChunk; ++c) {
-          const int j = c0 + lane + 32 * c;
-          v1[c] = j < ld ? W[(size_t)i * ld + j] : 0.0;
-          v2[c] = (has2 && j < ld) ? W[(size_t)i2 * ld + j] : 0.0;
-        }
-        const double f1 = (i != k) ? colk[i] : 0.0;
-        const double f2 = (has2 && i2 != k) ? colk[i2] : 0.0;
-#pragma unroll
-        for (int c = 0; c < kGjChunk; ++c) {
-          v1[c] = fma(-f1, rk[c], v1[c]);
-          v2[c] = fma(-f2, rk[c], v2[c]);
-        }
-#pragma unroll
-        for (int c = 0; c < kGjChunk; ++c) {
-          const int j = c0 + lane + 32 * c;
-          if (j < ld) {
-            if (i != k) W[(size_t)i * ld + j] = v1[c];
-            if (has2 && i2 != k) W[(size_t)i2 * ld + j] = v2[c];
-          }
-        }
-      }
-    }
+    gj_step<NT>(W, L, ld, k + 1, ncol, colk, k, false);
     __syncthreads();
   }
   return 0;
@@ -169,7 +207,7 @@ __device__ double recompute_green(const GridConst& gc, const int8_t* s, T* Gup, 
       }
     }
     __syncthreads();
-    if (gj_eliminate<NT>(W, L, red, redi, s_inv, s_piv, colk) != 0) {
+    if (gj_eliminate<NT>(W, L, ld, ld, red, redi, s_inv, s_piv, colk) != 0) {
       if (tid == 0) atomicOr(status_word, kStatusSingular);
       return -1.0;
     }
@@ -201,55 +239,18 @@ __device__ double recompute_green(const GridConst& gc, const int8_t* s, T* Gup, 
 template <int NT>
 __device__ int gj_invert_inplace(double* B, int L, double* red, int* redi, double* s_inv, int* s_piv,
                                  double* colk, int* perm) {
-  constexpr int kGjChunk = gj_chunk<NT>();
-  constexpr int NW = NT / 32;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   const int ld = L;
   for (int k = 0; k < L; ++k) {
-    double best = -1.0;
-    int bi = L;
-    for (int i = k + tid; i < L; i += NT) {
-      const double v = fabs(B[(size_t)i * ld + k]);
-      if (v > best) {
-        best = v;
-        bi = i;
-      }
-    }
-    for (int o = 16; o; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > best || (ov == best && oi < bi)) {
-        best = ov;
-        bi = oi;
-      }
-    }
-    if (lane == 0) {
-      red[warp] = best;
-      redi[warp] = bi;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      double b = red[0];
-      int p = redi[0];
-      for (int w = 1; w < NW; ++w)
-        if (red[w] > b || (red[w] == b && redi[w] < p)) {
-          b = red[w];
-          p = redi[w];
-        }
-      if (!(b > 0.0) || p >= L) {
-        *s_piv = -1;
-      } else {
-        *s_piv = p;
-        *s_inv = 1.0 / B[(size_t)p * ld + k];
-        perm[k] = p;
-      }
-    }
-    __syncthreads();
+    gj_pivot<NT>(B, L, ld, k, red, redi, s_inv, s_piv);
     const int p = *s_piv;
     if (p < 0) return -1;
+    if (tid == 0) perm[k] = p;
     const double inv = *s_inv;
-    // swap rows k and p, scale the new row k (its column-k entry becomes
-    // 1/pivot: the identity column folded in); record column k of the rest
+    // record column k; swap rows k and p, scale the new row k (its column-k
+    // entry becomes 1/pivot: the identity column folded in)
+    for (int i = tid; i < L; i += NT)
+      if (i != k && i != p) colk[i] = B[(size_t)i * ld + k];
     for (int j = tid; j < ld; j += NT) {
       const double a = B[(size_t)k * ld + j];
       const double b = B[(size_t)p * ld + j];
@@ -257,46 +258,10 @@ __device__ int gj_invert_inplace(double* B, int L, double* red, int* redi, doubl
       B[(size_t)k * ld + j] = (j == k) ? inv : b * inv;
       if (j == k) colk[p] = a;
     }
-    for (int i = tid; i < L; i += NT)
-      if (i != k && i != p) colk[i] = B[(size_t)i * ld + k];
     __syncthreads();
-    // eliminate: row i -= f_i * row k over all columns (column k of row i
-    // starts from 0, the identity column)
-    const double* bk = B + (size_t)k * ld;
-    for (int c0 = 0; c0 < ld; c0 += 32 * kGjChunk) {
-      double rk[kGjChunk];
-#pragma unroll
-      for (int c = 0; c < kGjChunk; ++c) {
-        const int j = c0 + lane + 32 * c;
-        rk[c] = j < ld ? bk[j] : 0.0;
-      }
-      for (int i = warp; i < L; i += 2 * NW) {
-        const int i2 = i + NW;
-        const bool has2 = i2 < L;
-        double v1[kGjChunk], v2[kGjChunk];
-#pragma unroll
-        for (int c = 0; c < kGjChunk; ++c) {
-          const int j = c0 + lane + 32 * c;
-          v1[c] = (j < ld && j != k) ? B[(size_t)i * ld + j] : 0.0;
-          v2[c] = (has2 && j < ld && j != k) ? B[(size_t)i2 * ld + j] : 0.0;
-        }
-        const double f1 = (i != k) ? colk[i] : 0.0;
-        const double f2 = (has2 && i2 != k) ? colk[i2] : 0.0;
-#pragma unroll
-        for (int c = 0; c < kGjChunk; ++c) {
-          v1[c] = fma(-f1, rk[c], v1[c]);
-          v2[c] = fma(-f2, rk[c], v2[c]);
-        }
-#pragma unroll
-        for (int c = 0; c < kGjChunk; ++c) {
-          const int j = c0 + lane + 32 * c;
-          if (j < ld) {
-            if (i != k) B[(size_t)i * ld + j] = v1[c];
-            if (has2 && i2 != k) B[(size_t)i2 * ld + j] = v2[c];
-          }
-        }
-      }
-    }
+    // row i -= f_i * row k over all columns (column k of row i starts from 0,
+    // the identity column)
+    gj_step<NT>(B, L, ld, 0, ld, colk, k, true);
     __syncthreads();
   }
   // undo the row interchanges as column interchanges, last first; a thread
