@@ -362,7 +362,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
 // Allocates kTmemCols TMEM columns (warp 0) and initialises the MMA
 // completion mbarrier s_mbar[0] and the refinement's eleven, s_mbar[1..11]
 // (the four "full" ones, 2 to 5, take one arrival per lane quarter and block of
-// eight contraction rows).
+// eight contraction rows, the four "consumed" ones, 6 to 9, one per issuing warp).
 __device__ inline void tc_setup(TcState* tc, uint32_t* s_tmem, unsigned long long* s_mbar,
                                 int* status) {
   (void)status;
@@ -375,7 +375,7 @@ __device__ inline void tc_setup(TcState* tc, uint32_t* s_tmem, unsigned long lon
   }
   if (threadIdx.x == 0) {
     for (int b = 0; b < 12; ++b)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(s_mbar + b)), "r"(b >= 2 && b <= 5 ? 8 : 1)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(s_mbar + b)), "r"(b >= 2 && b <= 5 ? 8 : b >= 6 && b <= 9 ? 2 : 1)
                    : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -426,10 +426,13 @@ __device__ __forceinline__ void bulk_wait0() { asm volatile("cp.async.bulk.wait_
 __device__ __forceinline__ void stage_group(const float* W, int nb, int nN, bool doW, const float* U, int mg,
                                             int ub, bool doU, int L, int KP, int j, int KS, float sw, float su,
                                             unsigned char* stage, size_t tile_bytes) {
-  const int cpt = kTileN * (KS / 8);  // 16-byte chunks per tile
-  const int nt = (doW ? 1 : 0) + (doU ? ub : 0);
-  for (int c = threadIdx.x; c < nt * cpt; c += kDelNT) {
-    const int t = c / cpt, cc = c - t * cpt;
+  // 128 threads take a tile's rows (a quarter-warp writes one 128-byte core
+  // matrix, conflict-free), the four groups of 128 the 16-byte chunks of K of
+  // all tiles in turn: one division by KS/8 per chunk and none per row
+  const int nk = KS / 8, nt = (doW ? 1 : 0) + (doU ? ub : 0);
+  const int r = threadIdx.x & (kTileN - 1);
+  for (int g = threadIdx.x / kTileN; g < nt * nk; g += kDelNT / kTileN) {
+    const int t = g / nk, m0 = (g - t * nk) * 8;
     const bool isW = doW && t == 0;
     const int u = t - (doW ? 1 : 0);
     const float* P = isW ? W : U;
@@ -437,11 +440,6 @@ __device__ __forceinline__ void stage_group(const float* W, int nb, int nN, bool
     const int nrows = isW ? nN : min(kTileN, L - row0);
     const float sc = isW ? sw : su;
     unsigned char* hi = isW ? stage : stage + (size_t)(2 + 2 * u) * tile_bytes;
-    // cc = ((row group * KS/8) + k chunk) * 8 + row within group: eight lanes
-    // write one 128-byte core matrix, conflict-free
-    const int r8 = cc & 7, rest = cc >> 3;
-    const int kc = rest % (KS / 8), grp = rest / (KS / 8);
-    const int r = grp * 8 + r8, m0 = kc * 8;
     // two 16-byte loads per chunk (rows are 16-byte aligned: KP % 4 == 0);
     // the second only below j <= KP - 4, so never past the row
     float4 xa = make_float4(0.f, 0.f, 0.f, 0.f), xb = xa;
@@ -626,13 +624,22 @@ __device__ __forceinline__ void flush_tiles(TcState* tc, float* Gu, float* Gd, i
             for (int c = 0; c < 8 / (kDelNT / 128); ++c) {
               const int cb = (128 / (kDelNT / 128)) * half + 16 * c;
               if (cb < N16) {  // warp-uniform: tcgen05.ld is issued by whole warps
-                float v[16];
+                float v[16], o[16];
                 tmem_ld16(tc->tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(u * kTileN + cb), v);
-                if (m < nN) {
-                  float* g = G + (size_t)(mb + cb) * ld + nb + m;
+                float* g = G + (size_t)(mb + cb) * ld + nb + min(m, nN - 1);
+                // all loads before the first store, and no condition per entry
+                // where the sixteen rows all exist
+                if (cb + 16 <= nM) {
+#pragma unroll
+                  for (int q = 0; q < 16; ++q) o[q] = g[(size_t)q * ld];
+                  if (m < nN) {
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) g[(size_t)q * ld] = fmaf(v[q], ds, o[q]);
+                  }
+                } else if (m < nN) {
 #pragma unroll
                   for (int q = 0; q < 16; ++q)
-                    if (cb + q < nM) g[(size_t)q * ld] += v[q] * ds;
+                    if (cb + q < nM) g[(size_t)q * ld] = fmaf(v[q], ds, g[(size_t)q * ld]);
                 }
               }
             }
@@ -861,23 +868,28 @@ __device__ inline void measure_rows(const float* Gu, const float* Gd, int ld, in
 // The same sums for G in shared memory (odd row pitch ld): thread k walks the
 // wrapped diagonal k of both spins in registers; for a fixed l the threads
 // of a warp read rows l+k at stride ld, i.e. 32 different banks.
+// A thread per diagonal and spin, the loads of eight terms before their
+// additions (in order).
 template <int NSP = 2>
 __device__ inline void measure_diagonals(const float* Gu, const float* Gd, int ld, int L, float* out) {
-  for (int k = threadIdx.x; k < L; k += kDelNT) {
-    float su = 0.f, sd = 0.f;
-    int l = 0;
-    for (; l + k < L; ++l) {
-      const int o = (l + k) * ld + l;
-      su += Gu[o];
-      if (NSP == 2) sd += Gd[o];
+  for (int e = threadIdx.x; e < NSP * L; e += kDelNT) {
+    const int k = e < L ? e : e - L;
+    const float* G = e < L ? Gu : Gd;
+    float sum = 0.f;
+    for (int l0 = 0; l0 < L; l0 += 8) {
+      float x[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        const int l = min(l0 + t, L - 1), r = l + k;
+        x[t] = G[(r < L ? r : r - L) * ld + l];
+      }
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        const int l = l0 + t;
+        sum += l >= L ? 0.f : l + k < L ? x[t] : -x[t];
+      }
     }
-    for (; l < L; ++l) {
-      const int o = (l + k - L) * ld + l;
-      su -= Gu[o];
-      if (NSP == 2) sd -= Gd[o];
-    }
-    out[k] = su;
-    if (NSP == 2) out[L + k] = sd;
+    out[e] = sum;
   }
   __syncthreads();
 }

@@ -47,12 +47,12 @@
 //     sigma s_j = +1; rows with sigma s_i = -1 get (A_ii difference) x H'_in
 //     added to V in the read-out, from the same slices of H'_in with the same
 //     products p + q <= 5 dropped, so V is the one of the sliced product.
-//   * H'^T is the other operand, cut from G by 15 warps straight into TMEM
+//   * H'^T is the other operand, cut from G by 14 warps straight into TMEM
 //     (the A operand of tcgen05.mma may live there): the tensor cores then
 //     read only A's slices, 2 KiB per MMA, from shared memory, and a 128 x 64
 //     x 16 MMA runs at its 32 cycles (measured alone: 32.1; with both operands
 //     in shared memory 48).  Four TMEM buffers of one K step of 16 each; the
-//     cutting warps and the issuing warp meet on mbarriers, there is no CTA
+//     cutting warps and the two issuing warps meet on mbarriers, there is no CTA
 //     barrier in the loop.
 // The update H' E only needs FP32 accuracy (|E| is small): split FP16
 // hi/lo parts with power-of-two scales, three products, FP32 accumulation,
@@ -61,11 +61,13 @@
 //
 // SM cycles per refinement of one spin at Lambda = 240 (phase timers in a copy
 // of the kernel), with A's slices streamed from L2 and H' cut into shared
-// memory, and as it is here: residual product 180k -> 132k (its MMAs alone
-// take 69k; what is above is the hand-over between the cutting warps and the
-// issuer, 50 cycles an MMA), its read-outs 50k -> 42k, update product 46k ->
-// 34k, its read-out 31k -> 26k, scale pass 16k -> 13k; at Lambda = 500 in all
-// 2.83M -> 1.98M.
+// memory, and as it is here: residual product 180k -> 117k (its MMAs alone
+// take 69k; what is above is the hand-over between the cutting and the issuing
+// warps), its read-outs 50k -> 39k, update product 46k -> 34k, its read-out
+// 31k -> 26k, scale pass 16k -> 13k; at Lambda = 500 in all 2.83M -> 1.85M.
+// Measured and not kept for Lambda > 256: H' and E^T written once as FP16
+// parts and staged by bulk copies (the chains' working set is beyond L2 there:
+// 673k cycles for the update product instead of 495k).
 //
 // max |E| over the matrix decides: above rc.emax_step (2^-8 by default) the
 // step is not taken and the caller recomputes G from scratch (Gauss-Jordan);
@@ -73,6 +75,8 @@
 // change of an entry over the steps.
 #pragma once
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "hfq_delayed.cuh"
 #include "hfq_device.cuh"
@@ -88,7 +92,13 @@ constexpr int kRfBufs = 4;
 constexpr int kRfBufCol = kRfLevels * kRfN;
 constexpr int kRfBufCols = kRfSlicesH * 8;
 static_assert(kRfBufCol + kRfBufs * kRfBufCols <= kTmemCols, "accumulators and H' buffers must fit the TMEM allocation");
-constexpr int kRfIssueWarp = 15;  // its elected lane issues every MMA; the other warps cut H'
+// Warps 14 and 15 issue the MMAs (one elected lane each), the others cut H'.
+// Two, on two schedulers, because each shares its scheduler with three cutting
+// warps: one alone took 50 cycles an MMA, which runs in 32.  The residual
+// product's levels are dealt out as 5, 4, 0 and 3, 2, 1 (nine products a K step
+// each), so that every accumulator belongs to one of them.
+constexpr int kRfIssueWarp = 15, kRfIssuers = 2;
+__host__ __device__ constexpr int rf_issuer_of(int level) { return level == 0 || level >= 4 ? 0 : 1; }
 constexpr int kRfAhead = 2;       // K steps of the next tile cut before a tile's read-out
 
 // K-major core-matrix layout of the update product's chunks (8 rows x 16
@@ -347,13 +357,14 @@ __device__ __forceinline__ float rf_product(RfPar& P, const unsigned char* sm, i
   const uint32_t bar_full = P.cbar + 8u, bar_empty = bar_full + 8u * kRfBufs;
   const uint32_t lane_base = P.tmem + ((uint32_t)(32 * q4) << 16);
   const float* fs = reinterpret_cast<const float*>(sm + rf_tab_bytes(L));
-  const int stride = q4 == (kRfIssueWarp & 3) ? NW / 4 - 1 : NW / 4;
+  const bool issuer = warp > kRfIssueWarp - kRfIssuers;
+  const int stride = q4 > (kRfIssueWarp & 3) - kRfIssuers ? NW / 4 - 1 : NW / 4;
   const int total = nmb * nib * NJ;
   float emax = 0.f;
   int vb = g4, vt = 0, vm = 0;  // the warp's next block: block of its tile, row tile, column block
   int v = g4;                   // ... and its place in the stream
   for (int tile = 0; tile < nmb * nib; ++tile) {
-    if (warp != kRfIssueWarp) {
+    if (!issuer) {
       // cut in registers, then stored once the buffer is free, so that little
       // is left to do between a buffer's release and its refill; the loads of
       // the warp's next block are issued before the cut.  A block: eight rows
@@ -434,17 +445,24 @@ __device__ __forceinline__ float rf_product(RfPar& P, const unsigned char* sm, i
         tc_fence_after();
         const uint32_t a0 = tm + kRfBufCol + nu % kRfBufs * kRfBufCols;
         const uint64_t bd = (desc & 0xffffffff00000000ull) | bk;
-        if (live) {
+        auto issue = [&](auto which) {
 #pragma unroll
           for (int q = 0; q < kRfSlicesH; ++q)
 #pragma unroll
             for (int p = 0; p + q < kRfLevels; ++p)
-              tc_mma_f16_ts(el, tm + (uint32_t)((p + q) * kRfN), a0 + (uint32_t)(q * 8), bd + (uint64_t)((uint32_t)p * slice),
-                            idesc, q > 0 || k > 0 ? 1 : 0);
+              if (rf_issuer_of(p + q) == decltype(which)::value)
+                tc_mma_f16_ts(el, tm + (uint32_t)((p + q) * kRfN), a0 + (uint32_t)(q * 8),
+                              bd + (uint64_t)((uint32_t)p * slice), idesc, q > 0 || k > 0 ? 1 : 0);
+        };
+        if (live) {
+          if (warp == kRfIssueWarp)
+            issue(std::integral_constant<int, 0>());
+          else
+            issue(std::integral_constant<int, 1>());
         }
         tc_commit_el(el, bar_e + 8u * (nu % kRfBufs));
       }
-      // the last step's products (the issuer has seen every use before it consumed)
+      // the last step's products (the issuers have seen every use before it consumed)
       const uint32_t nl = c0 + nk - 1u;
       if (live) live = rf_wait_warp(bar_e + 8u * (nl % kRfBufs), (nl / kRfBufs) & 1u);
       W.bad = !live;

@@ -20,8 +20,12 @@
 // shuffle, and right away evaluates slice r as the next proposal (flip ratio
 // from the new diagonals, Philox uniform drawn at the start of the sweep).
 // Rejections change nothing, so the next accepted slice is the lowest r > l
-// that accepts: a warp ballot and a shared-memory atomicMin find it, and one
-// barrier per accepted flip publishes it with its flip factors.
+// that accepts: every warp leaves the lowest of its rows, with its diagonal, in
+// a slot of its own, and after one barrier per accepted flip each warp takes
+// the minimum of the slots and each thread divides for its flip factor while
+// G's column and row are on their way.  (With one atomicMin for all warps, the
+// division before the barrier and a branch around every load, 256 chains at
+// Lambda = 100 took 86 ms for 550 sweeps; they take 75.)
 #include "hfq_delayed.cuh"
 #include "hfq_device.cuh"
 #include "hfq_gj.cuh"
@@ -43,7 +47,7 @@ struct SweepPos {
   long long t0;             // global index of the call's first sweep
   uint32_t sw;
   int l, par;
-  float fu, fd;
+  float f[2];               // flip factors of slice l (threads of spin up, of spin down)
 };
 // What its recomputes have added up to
 struct RecTotals {
@@ -81,6 +85,19 @@ struct ChainView {
   }
 };
 
+// The fallback and the contexts that do not refine: out of line, it is rare or
+// long, and its FP64 registers are not the sweep's.
+__device__ __noinline__ double recompute_from_scratch(unsigned char* smem, float* Gu, float* Gd, int ld, int n_spins,
+                                                      double* red, int* redi, double* s_inv, int* s_piv, int* status) {
+  const ChainConst& c = *reinterpret_cast<const ChainConst*>(smem + kChainOff);
+  // FP64 workspace in HBM, inverted by panels whose scratch overlays the idle
+  // part of shared memory (never G)
+  return recompute_green_inv<float, kDelNT, true>(
+      c.gc, reinterpret_cast<const int8_t*>(smem + c.lay.off_s), Gu, Gd, ld, c.ip.ws, red, redi, s_inv, s_piv,
+      reinterpret_cast<double*>(smem + c.lay.off_colk), reinterpret_cast<int*>(smem + c.lay.off_perm), true, status, 0,
+      n_spins, reinterpret_cast<double*>(smem + c.lay.off_gjb));
+}
+
 // A chain runs as stretches of sweeping between recomputes.  Everything a
 // stretch needs is re-derived at its start -- the field from shared memory,
 // the uniforms from Philox, the diagonal from G, the rest from SweepPos -- so
@@ -109,7 +126,6 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
   __shared__ int redi[NW];
   __shared__ double s_inv;
   __shared__ int s_piv, s_item;
-  __shared__ int s_next[3];  // next accepted slice, triple-buffered (see take_next)
   __shared__ int s_bad;
   __shared__ uint32_t s_tmem_base;
   __shared__ __align__(8) unsigned long long s_mbar[12];
@@ -142,22 +158,19 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
     __syncthreads();
     {
     const ChainView v(s_chain, smem);
-    const GridConst& gc = v.gc;
     const ItemPtrs& ip = v.ip;
-    const DelLayout& lay = v.lay;
     const int L = v.L, ld = v.ld;
     const bool resident = v.resident;
-    float *const Ggl = v.Ggl, *const Gu = v.Gu, *const Gd = v.Gd;
+    float *const Ggl = v.Ggl, *const Gu = v.Gu;
     int8_t* const ss = v.ss;
     if (resident) {
       for (int i = warp; i < (kMirror ? 1 : 2) * L; i += NW)
         for (int jj = lane; jj < L; jj += 32) Gu[(size_t)i * ld + jj] = Ggl[(size_t)i * L + jj];
     }
     for (int l = tid; l < L; l += NT) ss[l] = ip.s[l];
-    if (tid < 3) s_next[tid] = kNoSlice;
     if (tid == 0) {
       s_bad = 0;
-      s_pos = SweepPos{ip.cnt->accepted, ip.cnt->hash, ip.cnt->t, 0u, -1, 0, 0.f, 0.f};
+      s_pos = SweepPos{ip.cnt->accepted, ip.cnt->hash, ip.cnt->t, 0u, -1, 0, {0.f, 0.f}};
       s_rec = RecTotals{ip.cnt->drift, 0, 0};
     }
     __syncthreads();
@@ -179,7 +192,11 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
     float* dtile = gc.gtile ? reinterpret_cast<float*>(smem + lay.off_gtile) : nullptr;
     float* Pu = reinterpret_cast<float*>(smem + lay.off_U);  // [2][L][KP] (spin stride padded): U panels
     float* Pw = reinterpret_cast<float*>(smem + lay.off_W);  // [2][L][KP]: W panels
-    float* fac = reinterpret_cast<float*>(smem + lay.off_diag);  // [L][2]: flip factors of candidates
+    // [2][warps that own rows]: each warp's lowest accepting slice, G_up's and
+    // G_dn's diagonal there and its field, by rounds of two
+    int4* slots = reinterpret_cast<int4*>(smem + lay.off_diag);
+    const int nwa = min(NW, (L + 15) >> 4);
+    const bool active = warp < nwa;  // this warp owns rows (warp-uniform)
     unsigned char* stage = smem + lay.off_stage;
     const int KP = lay.KP;
     const int panel_floats4 = del_panel_floats(L, KP, kMirror ? 1 : 2) / 4;  // one panel, the kept spins
@@ -214,8 +231,8 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
     };
     uint32_t sw = s_pos.sw;
     int l = s_pos.l;  // next accepted slice; -1: the sweep begins
-    int par = s_pos.par;  // s_next buffer of the current round
-    float fu = s_pos.fu, fd = s_pos.fd;  // its flip factors
+    int par = s_pos.par;  // slots of the current round
+    float f = s_pos.f[tid & 1];  // its flip factor, of this thread's spin
     auto draw_uniforms = [&](long long t) {
 #pragma unroll
       for (int qq = 0; qq < kRowsPerThread; ++qq) {
@@ -265,11 +282,13 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
     };
 
     // Evaluates the owned slices r >= lo as proposals with the current
-    // diagonals of both spins (partner threads swap theirs); the lowest
-    // accepting slice of the CTA lands in s_next[par] (read after the next
-    // barrier), its flip factors in fac[2r], fac[2r+1].
+    // diagonals of both spins (partner threads swap theirs); the warp's lowest
+    // accepting slice goes to its slot of this round (read after the next
+    // barrier; written again only after the barrier that follows).
     auto propose = [&](int lo) {
-      int cand = kNoSlice;
+      if (!active) return;
+      int cand = kNoSlice, own = 0, cs = 0;
+      float cgu = 0.f, cgd = 0.f;
 #pragma unroll
       for (int qq = 0; qq < kRowsPerThread; ++qq) {
         if (qq * kRowStride >= L) break;  // uniform: rows beyond the grid
@@ -283,32 +302,34 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
           gu = sp ? other : dg[qq];
           gd = sp ? dg[qq] : other;
         }
-        bool acc = false, bad = false;
-        if (r < L && r >= lo) {
-          acc = del_decide(d0, d1, gu, gd, sv[qq], uv[qq], rule, &bad);
-          if (acc && sp == 0) {
-            float fu, fd;
-            del_factors(d0, d1, gu, gd, sv[qq], &fu, &fd);
-            fac[2 * r] = fu;
-            fac[2 * r + 1] = fd;
-          }
-        }
-        lastbad[qq] = bad && sp == 0;
+        bool bad;
+        const bool in = r < L && r >= lo;
+        const bool acc = del_decide(d0, d1, gu, gd, sv[qq], uv[qq], rule, &bad) && in;
+        lastbad[qq] = bad && in && sp == 0;
         const unsigned b = __ballot_sync(0xffffffffu, acc) & 0x55555555u;
-        if (b && cand == kNoSlice) cand = qq * kRowStride + warp * 16 + ((__ffs(b) - 1) >> 1);
+        if (b && cand == kNoSlice) {  // warp-uniform
+          own = __ffs(b) - 1;
+          cand = qq * kRowStride + warp * 16 + (own >> 1);
+          cgu = gu;
+          cgd = gd;
+          cs = sv[qq];
+        }
       }
-      if (lane == 0 && cand != kNoSlice) atomicMin(&s_next[par], cand);
+      if (lane == own) slots[par * nwa + warp] = make_int4(cand, __float_as_int(cgu), __float_as_int(cgd), cs);
     };
 
-    // After the barrier of a round: read the decision and reset the buffer
-    // that the round before used (every thread has read it before reaching
-    // this round's barrier, and it is written again only two rounds later).
-    // Also counts the bad ratios among the proposals this round decided,
-    // i.e. the owned slices in [lo, next].
+    // After the barrier of a round: the lowest of the slots, and this thread's
+    // flip factor Delta / R (its spin's; spin up's for a mirrored sweep).  Also
+    // counts the bad ratios among the proposals this round decided, i.e. the
+    // owned slices in [lo, next].
     auto take_next = [&](int lo) -> int {
-      const int nxt = s_next[par];
-      if (tid == 0) s_next[(par + 2) % 3] = kNoSlice;
-      par = (par + 1) % 3;
+      const int4* round = slots + par * nwa;
+      const int nxt = __reduce_min_sync(0xffffffffu, round[min(lane, nwa - 1)].x);
+      const int4 w = round[nxt < L ? (nxt >> 4) & (NW - 1) : 0];
+      par ^= 1;
+      const bool plus = (w.w > 0) == (kMirror || sp == 0);
+      const float del = plus ? d0 : d1, g = __int_as_float(kMirror || sp == 0 ? w.y : w.z);
+      f = del / __fadd_rn(1.f, __fmul_rn(__fsub_rn(1.f, g), del));
       const int hi = nxt < L ? nxt : L - 1;
 #pragma unroll
       for (int qq = 0; qq < kRowsPerThread; ++qq) {
@@ -325,113 +346,89 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
         propose(0);
         __syncthreads();
         l = take_next(0);
-        // flip factors of the accepted slice; read before any flush or
-        // recompute, whose shared-memory workspace may overlay fac[]
-        if (l < L) {
-          fu = fac[2 * l];
-          fd = fac[2 * l + 1];
-        }
       }
       while (l < L) {
-        if constexpr (kMirror) {
-          // spin up only: the even thread of a pair appends u_i (column l),
-          // the odd one w_i (row l); one shuffle gives both the pair's values
-          float gq[kRowsPerThread];
+        if (active) {
+          // base G entries of every owned row first (before any panel store), so
+          // their latency -- L2 when G lives in HBM -- overlaps the dot products.
+          // Rows beyond the grid repeat the last one and store nothing; no load
+          // sits behind a branch.
+          float gc_q[kRowsPerThread], gr_q[kRowsPerThread];  // column / row entry (mirrored: the thread's one of them)
+          auto base_entries = [&](const float* g, int gld) {
 #pragma unroll
-          for (int qq = 0; qq < kRowsPerThread; ++qq) {
-            if (qq * kRowStride >= L) break;  // uniform: rows beyond the grid
-            const int i = row0 + qq * kRowStride;
-            gq[qq] = i < L ? (sp ? Gs[l * ld + i] : Gs[i * ld + l]) : 0.f;
-          }
-#pragma unroll
-          for (int qq = 0; qq < kRowsPerThread; ++qq) {
-            if (qq * kRowStride >= L) break;  // uniform: rows beyond the grid
-            const int i = row0 + qq * kRowStride;
-            const int oi = i * KP, ol = l * KP;  // 32-bit shared-memory offsets
-            float c4[4] = {0.f, 0.f, 0.f, 0.f};
-            if (i < L) {
-              // even lane: U row i . W row l; odd lane: W row i . U row l.  The
-              // first load reads a distinct row in every lane (U or W, whose
-              // rows of one index sit 16 banks apart), the second the pair's
-              // two shared rows: both conflict-free
-              const float4* Ar = reinterpret_cast<const float4*>((sp ? Ws : Us) + oi);
-              const float4* Br = reinterpret_cast<const float4*>((sp ? Us : Ws) + ol);
-              const int j4 = (j + 3) >> 2;
-              for (int m4 = 0; m4 < j4; ++m4) {
-                const float4 a1 = Ar[m4], b1 = Br[m4];
-                c4[0] = __fmaf_rn(a1.x, b1.x, c4[0]);
-                c4[1] = __fmaf_rn(a1.y, b1.y, c4[1]);
-                c4[2] = __fmaf_rn(a1.z, b1.z, c4[2]);
-                c4[3] = __fmaf_rn(a1.w, b1.w, c4[3]);
-              }
-            }
-            const float dot = gq[qq] + ((c4[0] + c4[1]) + (c4[2] + c4[3]));
-            const float mine = i >= L ? 0.f : sp ? dot * fu : dot - ((i == l) ? 1.f : 0.f);
-            const float theirs = __shfl_xor_sync(0xffffffffu, mine, 1);
-            if (i < L) {
-              const float uu = sp ? theirs : mine, ww = sp ? mine : theirs;
-              if (sp) {
-                exq = __vmaxu4(exq, ((__float_as_uint(ww) << 1) >> 24) << 8);
-                Ws[oi + j] = ww;
+            for (int qq = 0; qq < kRowsPerThread; ++qq) {
+              if (qq * kRowStride >= L) break;  // uniform: rows beyond the grid
+              const int i = min(row0 + qq * kRowStride, L - 1);
+              if constexpr (kMirror) {
+                gc_q[qq] = g[sp ? l * gld + i : i * gld + l];
               } else {
-                exq = __vmaxu4(exq, (__float_as_uint(uu) << 1) >> 24);
-                Us[oi + j] = uu;
-              }
-              dg[qq] = __fmaf_rn(uu, ww, dg[qq]);
-              if (i == l) {
-                sv[qq] = -sv[qq];
-                if (sp == 0) ss[i] = (int8_t)sv[qq];
+                gc_q[qq] = g[i * gld + l];  // 2 L^2 < 2^31: 32-bit offsets
+                gr_q[qq] = g[l * gld + i];
               }
             }
-          }
-        } else {
-        // append column j of the panels for the owned rows of this thread's spin
-        const float f = sp ? fd : fu;
-        // base G entries of every owned row first (before any panel store), so
-        // their latency -- L2 when G lives in HBM -- overlaps the dot products
-        float gil_q[kRowsPerThread], gli_q[kRowsPerThread];
+          };
+          if (resident)
+            base_entries(reinterpret_cast<const float*>(smem + lay.off_G) + (sp && !kMirror ? L * ld : 0), ld);
+          else
+            base_entries(Ggl + (sp && !kMirror ? L * L : 0), L);
 #pragma unroll
-        for (int qq = 0; qq < kRowsPerThread; ++qq) {
-          if (qq * kRowStride >= L) break;  // uniform: rows beyond the grid
-          const int i = row0 + qq * kRowStride;
-          gil_q[qq] = i < L ? Gs[i * ld + l] : 0.f;  // 2 L^2 < 2^31: 32-bit offsets
-          gli_q[qq] = i < L ? Gs[l * ld + i] : 0.f;
-        }
-#pragma unroll
-        for (int qq = 0; qq < kRowsPerThread; ++qq) {
-          if (qq * kRowStride >= L) break;  // uniform: rows beyond the grid
-          const int i = row0 + qq * kRowStride;
-          if (i >= L) continue;
-          const float gil = gil_q[qq], gli = gli_q[qq];
-          float c4[4] = {0.f, 0.f, 0.f, 0.f}, r4[4] = {0.f, 0.f, 0.f, 0.f};
-          const int oi = i * KP, ol = l * KP;  // 32-bit shared-memory offsets
-          const float4* Ui = reinterpret_cast<const float4*>(Us + oi);
-          const float4* Wl = reinterpret_cast<const float4*>(Ws + ol);
-          const float4* Ul = reinterpret_cast<const float4*>(Us + ol);
-          const float4* Wi = reinterpret_cast<const float4*>(Ws + oi);
-          const int j4 = (j + 3) >> 2;
-          for (int m4 = 0; m4 < j4; ++m4) {
-            const float4 a1 = Ui[m4], b1 = Wl[m4], a2 = Ul[m4], b2 = Wi[m4];
-            c4[0] = __fmaf_rn(a1.x, b1.x, c4[0]);
-            c4[1] = __fmaf_rn(a1.y, b1.y, c4[1]);
-            c4[2] = __fmaf_rn(a1.z, b1.z, c4[2]);
-            c4[3] = __fmaf_rn(a1.w, b1.w, c4[3]);
-            r4[0] = __fmaf_rn(a2.x, b2.x, r4[0]);
-            r4[1] = __fmaf_rn(a2.y, b2.y, r4[1]);
-            r4[2] = __fmaf_rn(a2.z, b2.z, r4[2]);
-            r4[3] = __fmaf_rn(a2.w, b2.w, r4[3]);
+          for (int qq = 0; qq < kRowsPerThread; ++qq) {
+            if (qq * kRowStride >= L) break;  // uniform: rows beyond the grid
+            const int i0 = row0 + qq * kRowStride, i = min(i0, L - 1);
+            const int oi = i * KP, ol = l * KP;  // 32-bit shared-memory offsets
+            // the panels are zero past column j: whole groups of eight columns
+            const int j8 = (j + 7) >> 3;
+            float c4[4] = {0.f, 0.f, 0.f, 0.f};
+            auto dot = [&](const float4* x, const float4* y, float* acc) {
+#pragma unroll 1
+              for (int m = 0; m < j8; ++m) {
+                const float4 a1 = x[2 * m], b1 = y[2 * m], a2 = x[2 * m + 1], b2 = y[2 * m + 1];
+                acc[0] = __fmaf_rn(a1.x, b1.x, acc[0]);
+                acc[1] = __fmaf_rn(a1.y, b1.y, acc[1]);
+                acc[2] = __fmaf_rn(a1.z, b1.z, acc[2]);
+                acc[3] = __fmaf_rn(a1.w, b1.w, acc[3]);
+                acc[0] = __fmaf_rn(a2.x, b2.x, acc[0]);
+                acc[1] = __fmaf_rn(a2.y, b2.y, acc[1]);
+                acc[2] = __fmaf_rn(a2.z, b2.z, acc[2]);
+                acc[3] = __fmaf_rn(a2.w, b2.w, acc[3]);
+              }
+            };
+            if constexpr (kMirror) {
+              // spin up only: the even thread of a pair appends u_i (column l),
+              // the odd one w_i (row l); one shuffle gives both the pair's values.
+              // Even lane: U row i . W row l; odd lane: W row i . U row l.  The
+              // first operand reads a distinct row in every lane (U or W, whose
+              // rows of one index sit 16 banks apart), the second the pair's two
+              // shared rows: both conflict-free
+              float* mine_p = sp ? Ws : Us;
+              dot(reinterpret_cast<const float4*>(mine_p + oi), reinterpret_cast<const float4*>((sp ? Us : Ws) + ol), c4);
+              const float v = gc_q[qq] + ((c4[0] + c4[1]) + (c4[2] + c4[3]));
+              const float mine = sp ? v * f : v - ((i == l) ? 1.f : 0.f);
+              const float theirs = __shfl_xor_sync(0xffffffffu, mine, 1);
+              if (i0 < L) {
+                exq = __vmaxu4(exq, ((__float_as_uint(mine) << 1) >> 24) << (sp ? 8 : 0));
+                mine_p[oi + j] = mine;
+                dg[qq] = __fmaf_rn(mine, theirs, dg[qq]);
+              }
+            } else {
+              // append column j of the panels for the owned rows of this thread's spin
+              float r4[4] = {0.f, 0.f, 0.f, 0.f};
+              dot(reinterpret_cast<const float4*>(Us + oi), reinterpret_cast<const float4*>(Ws + ol), c4);
+              dot(reinterpret_cast<const float4*>(Us + ol), reinterpret_cast<const float4*>(Ws + oi), r4);
+              const float uu = gc_q[qq] + ((c4[0] + c4[1]) + (c4[2] + c4[3])) - ((i == l) ? 1.f : 0.f);
+              const float ww = (gr_q[qq] + ((r4[0] + r4[1]) + (r4[2] + r4[3]))) * f;
+              if (i0 < L) {
+                exq = __vmaxu4(exq, ((__float_as_uint(uu) << 1) >> 24) | (((__float_as_uint(ww) << 1) >> 24) << 8));
+                Us[oi + j] = uu;
+                Ws[oi + j] = ww;
+                dg[qq] = __fmaf_rn(uu, ww, dg[qq]);
+              }
+            }
+            if (i0 == l) {
+              sv[qq] = -sv[qq];
+              if (sp == 0) ss[i0] = (int8_t)sv[qq];
+            }
           }
-          const float uu = gil + ((c4[0] + c4[1]) + (c4[2] + c4[3])) - ((i == l) ? 1.f : 0.f);
-          const float ww = (gli + ((r4[0] + r4[1]) + (r4[2] + r4[3]))) * f;
-          exq = __vmaxu4(exq, ((__float_as_uint(uu) << 1) >> 24) | (((__float_as_uint(ww) << 1) >> 24) << 8));
-          Us[oi + j] = uu;
-          Ws[oi + j] = ww;
-          dg[qq] = __fmaf_rn(uu, ww, dg[qq]);
-          if (i == l) {
-            sv[qq] = -sv[qq];
-            if (sp == 0) ss[i] = (int8_t)sv[qq];
-          }
-        }
         }
         // the decision hash by the last thread (which owns no row for L <= 255)
         if (tid == NT - 1)
@@ -442,16 +439,8 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
         ++j;
         propose(l + 1);
         __syncthreads();
-        const int lnext = take_next(l + 1);
-        float fu_next = 0.f, fd_next = 0.f;
-        if (lnext < L) {
-          fu_next = fac[2 * lnext];
-          fd_next = fac[2 * lnext + 1];
-        }
+        l = take_next(l + 1);
         if (j == K) flush();
-        l = lnext;
-        fu = fu_next;
-        fd = fd_next;
         if (--left == 0) break;
       }
       if (left == 0) {
@@ -513,9 +502,8 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
       s_pos.sw = sw;
       s_pos.l = l;
       s_pos.par = par;
-      s_pos.fu = fu;
-      s_pos.fd = fd;
     }
+    if (tid < 2) s_pos.f[tid] = f;
     done = left != 0;
     recompute = left == 0 && gc.n_wrap > 0;
     }
@@ -532,8 +520,6 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
     const bool resident = v.resident;
     float *const Ggl = v.Ggl, *const Gu = v.Gu, *const Gd = v.Gd;
     int8_t* const ss = v.ss;
-    double* colk = reinterpret_cast<double*>(smem + lay.off_colk);
-    int* perm = reinterpret_cast<int*>(smem + lay.off_perm);
     double d = -1.0;
     // G in HBM while the refinement runs, where its staging overlays a
     // resident G (else it works on G where it lies)
@@ -569,12 +555,8 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
         ++s_rec.n_fb;
     }
     if (d < 0.0) {
-      // from scratch: FP64 workspace in HBM, inverted by panels whose
-      // scratch overlays the idle part of shared memory (never G)
-      d = recompute_green_inv<float, NT, true>(
-          gc, ss, in_hbm ? Ggl : Gu, in_hbm ? Ggl + (size_t)L * L : Gd, in_hbm ? L : ld, ip.ws, red, redi,
-          &s_inv, &s_piv, colk, perm, true, a.status, 0, kMirror ? 1 : 2,
-          reinterpret_cast<double*>(smem + lay.off_gjb));
+      d = recompute_from_scratch(smem, in_hbm ? Ggl : Gu, in_hbm ? Ggl + (size_t)L * L : Gd, in_hbm ? L : ld, kSpins, red,
+                                 redi, &s_inv, &s_piv, a.status);
     }
     if (in_hbm) {
       for (int i = warp; i < kSpins * L; i += NW)
@@ -590,12 +572,11 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
     }
 
     const ChainView v(s_chain, smem);
-    const GridConst& gc = v.gc;
     const ItemPtrs& ip = v.ip;
     const DelLayout& lay = v.lay;
     const int L = v.L, ld = v.ld;
     const bool resident = v.resident;
-    float *const Ggl = v.Ggl, *const Gu = v.Gu, *const Gd = v.Gd;
+    float *const Ggl = v.Ggl, *const Gu = v.Gu;
     int8_t* const ss = v.ss;
     if (resident) {
       for (int i = warp; i < (kMirror ? 1 : 2) * L; i += NW)
