@@ -304,7 +304,7 @@ int hfqmc_put_trace(hfqmc_ctx *ctx, int grid, const uint32_t *bits, int64_t n_wo
  * device work.  The call returns after its work on cuda_stream is done:
  * HFQMC_OK, HFQMC_ENUMERIC (zero pivot or non-finite G), HFQMC_ECUDA.
  *
- * Memory: the [A | M] workspace lives in shared memory while it fits (L <= 156),
+ * Memory: the [A | M] workspace lives in shared memory while it fits (L <= 159),
  * else with the bath matrix in one file-scope device array of 3 *
  * HFQMC_NOALLOC_MAX_L^2 doubles (1.5 MiB) that every GPU which loads the
  * library holds until the process exits (the status words are always there).

@@ -18,7 +18,7 @@
 //    panel in shared memory, two barriers per pivot column) on the chain's
 //    HBM workspace, which it reads and writes once per panel instead of once
 //    per pivot column -- the FP32 delayed path always, the initialisation
-//    whenever the panel fits.
+//    whenever the panel fits, there also with a cluster of CTAs per matrix.
 #pragma once
 #include "hfq_device.cuh"
 
@@ -306,23 +306,49 @@ __device__ int gj_invert_inplace(double* B, int L, double* red, int* redi, doubl
 // then the pivot rows' slab, pitch L); perm, pos: L ints each of shared
 // memory (pivot row of step k; step of row i).  Returns -1 on a zero pivot
 // (uniformly in all threads), 0 otherwise.
+//
+// kCluster: the np CTAs of a cluster invert one matrix, each calling this with
+// its part: every one reduces the panels (the same arithmetic in each), and
+// updates and stores its L / np columns, so every entry sees the operations of
+// the one-CTA form in the same order.  Two cluster barriers per panel: a panel
+// is overwritten only after every CTA has loaded it (arrive after the load,
+// wait before the store), and the next one is loaded only after every CTA has
+// stored its columns.  The panel is read from L2 (the columns of others); the
+// other reads are of the CTA's own columns.
 // ---------------------------------------------------------------------------
 
-template <int NT>
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+  cluster_arrive();
+  cluster_wait();
+}
+
+template <int NT, bool kCluster = false>
 __device__ int gj_invert_blocked(double* B, int L, double* red, int* redi, double* s_inv, int* s_piv,
-                                 int* perm, int* pos, double* pan) {
+                                 int* perm, int* pos, double* pan, int part = 0, int np = 1) {
   constexpr int NW = NT / 32;
   constexpr int KB = kGjPanel, PP = KB + 1;  // odd pitch: a column of the panel is conflict-free
   constexpr int TR = 8;                      // rows of an update item (one warp, 32 columns)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   double* slab = pan + (size_t)L * PP;
+  // the columns this CTA updates
+  const int jlo = kCluster ? (int)((long long)L * part / np) : 0;
+  const int jhi = kCluster ? (int)((long long)L * (part + 1) / np) : L;
   for (int i = tid; i < L; i += NT) pos[i] = -1;
   __syncthreads();
   for (int k0 = 0; k0 < L; k0 += KB) {
     const int bb = min(KB, L - k0);
     for (int i = warp; i < L; i += NW)
-      if (lane < bb) pan[i * PP + lane] = B[(size_t)i * L + k0 + lane];
+      if (lane < bb) pan[i * PP + lane] = kCluster ? __ldcg(B + (size_t)i * L + k0 + lane) : B[(size_t)i * L + k0 + lane];
     __syncthreads();
+    if constexpr (kCluster) cluster_arrive();  // this CTA has loaded the panel
     // the largest |pivot| (then the lowest row) among the unused rows,
     // compared as the magnitudes' bit patterns: for non-negative doubles
     // their order is that of unsigned integers, and the integer compares
@@ -390,7 +416,10 @@ __device__ int gj_invert_blocked(double* B, int L, double* red, int* redi, doubl
       // candidates of column t + 1 may overwrite them after it
       __syncthreads();
       const int p = *s_piv;
-      if (p < 0) return -1;
+      if (p < 0) {
+        if constexpr (kCluster) cluster_wait();  // the same panel, so every CTA of the cluster leaves here
+        return -1;
+      }
       const double inv = *s_inv;
       unsigned long long best = 0ull;
       int bi = L;
@@ -420,20 +449,22 @@ __device__ int gj_invert_blocked(double* B, int L, double* red, int* redi, doubl
     }
     // the pivot rows of the other columns, then their rank-b update, in
     // items of TR rows x 32 columns spread over the warps; the nR other
-    // columns are numbered c = 0 .. nR - 1 around the panel
+    // columns (of this CTA) are numbered c = 0 .. nR - 1 around the panel
     const int* pk = perm + k0;
-    for (int e = tid; e < bb * L; e += NT) {
-      const int t = e / L, j = e - t * L;
-      slab[e] = B[(size_t)pk[t] * L + j];
+    const int nj = jhi - jlo;
+    for (int e = tid; e < bb * nj; e += NT) {
+      const int t = e / nj, j = jlo + e - t * nj;
+      slab[t * L + j] = B[(size_t)pk[t] * L + j];
     }
     __syncthreads();
-    const int nR = L - bb;
+    const int plo = min(max(k0, jlo), jhi), phi = min(max(k0 + bb, jlo), jhi);
+    const int nL = plo - jlo, nR = nL + jhi - phi;
     const int ncg = (nR + 31) / 32, nrb = (L + TR - 1) / TR;
     for (int it = warp; it < ncg * nrb; it += NW) {
       const int cg = it % ncg, r0 = (it / ncg) * TR;
       const int c = cg * 32 + lane;
       const bool jin = c < nR;
-      const int j = c < k0 ? c : c + bb;
+      const int j = c < nL ? jlo + c : phi + c - nL;
       double acc[TR];
 #pragma unroll
       for (int q = 0; q < TR; ++q) {
@@ -454,9 +485,13 @@ __device__ int gj_invert_blocked(double* B, int L, double* red, int* redi, doubl
       for (int q = 0; q < TR; ++q)
         if (jin && r0 + q < L) B[(size_t)(r0 + q) * L + j] = acc[q];
     }
+    if constexpr (kCluster) cluster_wait();  // every CTA has loaded the panel
     for (int i = warp; i < L; i += NW)
-      if (lane < bb) B[(size_t)i * L + k0 + lane] = pan[i * PP + lane];
-    __syncthreads();
+      if (lane < bb && k0 + lane >= jlo && k0 + lane < jhi) B[(size_t)i * L + k0 + lane] = pan[i * PP + lane];
+    if constexpr (kCluster)
+      cluster_barrier();
+    else
+      __syncthreads();
   }
   return 0;
 }

@@ -27,10 +27,11 @@
 //     every partial sum is an integer below 2^24 for Lambda <= 512: the
 //     accumulation is exact, in any order).  Dropped levels and the slices'
 //     remainders leave |E - E_exact| ~ 1e-10 of |A||H'|.
-//   * The six level sums are combined exactly in integers,
-//     V = sum_l S_l 2^{7 (5 - l)}, so A H' = V 2^{ea + eh - 49}, and
-//     E = delta - V 2^{ea+eh-49} is formed as an integer before it is
-//     rounded to FP32: the cancellation costs nothing.
+//   * The six level sums combine as V = sum_l S_l 2^{7 (5 - l)}, so A H' =
+//     V 2^{ea + eh - 49}, and E = delta - V 2^{ea+eh-49} is exact before it is
+//     rounded to FP32: the cancellation costs nothing.  Near the inverse the
+//     leading levels cancel, so Horner's rule in FP32 is exact while its
+//     partial sums stay below 2^24 (checked); else 64-bit integers are used.
 //
 // The residual product on the tensor cores, E^T = 1 - H'^T A^T tile by tile
 // (128 columns n of H' = TMEM lanes, 64 rows i of A):

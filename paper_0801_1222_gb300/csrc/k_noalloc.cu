@@ -43,7 +43,7 @@ __host__ __device__ inline int noalloc_pitch(int L) { return (L + noalloc_cols(L
 __host__ __device__ inline size_t noalloc_smem(int L) {
   return ((size_t)L * noalloc_pitch(L) + L) * sizeof(double);
 }
-// whether a share's [A | M] fits in shared memory (L <= 156); else the
+// whether a share's [A | M] fits in shared memory (L <= 159); else the
 // workspace is the scratch array and one CTA does both spins
 inline bool noalloc_shared(int L) { return noalloc_smem(L) <= kSmemCap; }
 

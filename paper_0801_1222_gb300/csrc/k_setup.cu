@@ -164,6 +164,32 @@ int launch_refine_prep(int L, const double* Minv, double lambda, RefineConst* rc
   return (int)cudaGetLastError();
 }
 
+// The chain's accumulators zeroed; its counters too on the first bath.
+template <int NT>
+__device__ __forceinline__ void reset_chain(const ItemPtrs& ip, int L, int first_time) {
+  const int tid = threadIdx.x;
+  for (int k = tid; k < 2 * L; k += NT) ip.acc[k] = 0.0;
+  for (int k = tid; k < kBins * L; k += NT) ip.bins[k] = 0.0;
+  for (int k = tid; k < 1 + kBins; k += NT) ip.accD[k] = 0.0;
+  if (tid == 0) {
+    ChainCounters c;
+    if (first_time) {
+      c.t = 0;
+      c.proposals = 0;
+      c.accepted = 0;
+      c.recomputes = 0;
+      c.hash = kFnvOffset;
+      c.bad = 0;
+      c.status = 0;
+      c.fallbacks = 0;
+    } else {
+      c = *ip.cnt;
+    }
+    c.drift = 0.0;
+    *ip.cnt = c;
+  }
+}
+
 // Initial (or, after a new bath, rebuilt) Green matrices of every chain of a
 // grid: block (chain, spin), so the two spins of a chain are inverted by two
 // CTAs at once.  The spin-up block also resets the chain's accumulators.
@@ -202,26 +228,74 @@ __global__ void __launch_bounds__(256) k_init_chains(SweepArgs a, const GridCons
     recompute_green_inv<T, NT>(gc, sf, G, G + (size_t)L * L, L, W, red, redi, &s_inv, &s_piv, colk, perm,
                                false, a.status, sp, sp + 1);
   if (sp != 0) return;
-  for (int k = tid; k < 2 * L; k += NT) ip.acc[k] = 0.0;
-  for (int k = tid; k < kBins * L; k += NT) ip.bins[k] = 0.0;
-  for (int k = tid; k < 1 + kBins; k += NT) ip.accD[k] = 0.0;
-  if (tid == 0) {
-    ChainCounters c;
-    if (first_time) {
-      c.t = 0;
-      c.proposals = 0;
-      c.accepted = 0;
-      c.recomputes = 0;
-      c.hash = kFnvOffset;
-      c.bad = 0;
-      c.status = 0;
-      c.fallbacks = 0;
-    } else {
-      c = *ip.cnt;
+  reset_chain<NT>(ip, L, first_time);
+}
+
+// The same with the workspace in HBM, inverted by panels, np CTAs (a cluster)
+// per matrix with a share of the columns each.  Bound by the FP64 pipe (L^3
+// DFMA) of the SMs that have a CTA: 128 chains at L = 500 are 256 inversions on
+// 152 SMs, two waves of 37 ms, and 16 chains at L = 200 leave 120 SMs idle.  For
+// a particle-hole symmetric bath only spin up is inverted and G_dn = 1 - G_up^T
+// taken from the FP64 inverse before it is rounded (gridDim.y = 1): half the
+// work, and room for twice the CTAs per matrix.  hfqmc_set_G0 (the whole call):
+// L = 500, 128 chains 74.9 -> 37.8 ms; L = 240, 64 chains 4.4 -> 2.9; L = 200,
+// 16 chains 2.7 -> 1.4; L = 100, 256 chains 1.7 -> 0.95.  Every CTA reduces all
+// panels (the serial part), so np CTAs gain less than np times.
+template <typename T>
+__global__ void __launch_bounds__(256) k_init_chains_cluster(SweepArgs a, const GridConst* gptr, int item0,
+                                                             int first_time, int np) {
+  constexpr int NT = 256, NW = NT / 32;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  __shared__ double red[NW];
+  __shared__ int redi[NW];
+  __shared__ double s_inv;
+  __shared__ int s_piv;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sp = blockIdx.y;
+  const int part = blockIdx.x % np;
+  const ItemPtrs ip = a.items[item0 + blockIdx.x / np];
+  const GridConst gc = *gptr;
+  const int L = gc.L;
+  const bool mirror = gridDim.y == 1;
+  double* colk = reinterpret_cast<double*>(dsm);
+  int* perm = reinterpret_cast<int*>(colk + L);
+  int* pos = reinterpret_cast<int*>(colk);
+  int8_t* sf = reinterpret_cast<int8_t*>(perm + L);
+  double* W = ip.ws + (size_t)sp * L * L;
+  double* pan = reinterpret_cast<double*>(dsm + init_head_bytes(L));
+  for (int l = tid; l < L; l += NT) sf[l] = first_time ? initial_spin(l, ip.chain, ip.grid, a.seed) : ip.s[l];
+  __syncthreads();
+  // B = M^{-1} (1 + D) - D, a share of the rows each
+  const int sig = sp ? -1 : 1;
+  for (int i = part * NW + warp; i < L; i += np * NW) {
+    const double* Mi = gc.Minv + (size_t)i * L;
+    double* Wi = W + (size_t)i * L;
+    for (int j = lane; j < L; j += 32) {
+      const double d = (sig * (int)sf[j] > 0) ? gc.dV[0] : gc.dV[1];
+      __stcg(Wi + j, Mi[j] * (1.0 + d) - ((i == j) ? d : 0.0));
     }
-    c.drift = 0.0;
-    *ip.cnt = c;
   }
+  cluster_barrier();  // also: every CTA of the cluster has read the field
+  if (gj_invert_blocked<NT, true>(W, L, red, redi, &s_inv, &s_piv, perm, pos, pan, part, np) != 0) {
+    if (tid == 0 && part == 0) atomicOr(a.status, kStatusSingular);
+  } else {
+    T* G = reinterpret_cast<T*>(ip.G) + (size_t)sp * L * L;
+    T* Gd = reinterpret_cast<T*>(ip.G) + (size_t)L * L;
+    bool finite = true;
+    for (int i = part * NW + warp; i < L; i += np * NW) {
+      const double* Si = W + (size_t)perm[i] * L;
+      for (int j = lane; j < L; j += 32) {
+        const double gn = __ldcg(Si + pos[j]);
+        finite = finite && isfinite(gn);
+        G[(size_t)i * L + j] = (T)gn;
+        if (mirror) Gd[(size_t)j * L + i] = (T)((i == j ? 1.0 : 0.0) - gn);
+      }
+    }
+    if (!finite) atomicOr(a.status, kStatusNonFinite);
+  }
+  if (sp != 0 || part != 0) return;
+  if (first_time)
+    for (int l = tid; l < L; l += NT) ip.s[l] = sf[l];
+  reset_chain<NT>(ip, L, first_time);
 }
 
 size_t init_smem(int L, bool gj_smem) {
@@ -229,9 +303,45 @@ size_t init_smem(int L, bool gj_smem) {
 }
 
 int launch_init_chains(const SweepArgs& a, const GridConst* d_grid_ptr, int item0, int n_chains,
-                       int L, bool f64, bool first_time, bool gj_smem, cudaStream_t st) {
+                       int L, bool f64, bool first_time, bool gj_smem, bool has_U, bool mirror, cudaStream_t st) {
   const size_t sm = init_smem(L, gj_smem);
   cudaError_t e;
+  if (!gj_smem && init_blocked(L) && has_U) {
+    const int spins = mirror ? 1 : 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    // The most CTAs per matrix (a portable cluster) for which all matrices are
+    // worked on at once; more would queue behind each other.  np = 1 without
+    // the mirror leaves k_init_chains, whose panel loads need not go to L2 (50
+    // chains at L = 240, both spins: 4.3 ms against 4.7).
+    auto go = [&](auto* f) {
+      cudaError_t r = raise_smem_limit(f, sm);
+      if (r != cudaSuccess) return (int)r;
+      int np = 8;
+      for (; np > 1; np /= 2) {
+        if (L < 32 * np) continue;
+        at[0].val.clusterDim.x = np;
+        cfg.gridDim = dim3(n_chains * np, spins);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess) (void)cudaGetLastError();
+        if (n >= n_chains * spins) break;
+      }
+      if (np == 1 && !mirror) return -1;
+      at[0].val.clusterDim.x = np;
+      cfg.gridDim = dim3(n_chains * np, spins);
+      return (int)cudaLaunchKernelEx(&cfg, f, a, d_grid_ptr, item0, first_time ? 1 : 0, np);
+    };
+    const int r = f64 ? go(k_init_chains_cluster<double>) : go(k_init_chains_cluster<float>);
+    if (r >= 0) return r;
+  }
   if (f64) {
     e = cudaFuncSetAttribute(k_init_chains<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return (int)e;
