@@ -28,10 +28,11 @@ int launch_bath_inverse(int L, const double* M, double* Minv, int* status, cudaS
 int launch_refine_prep(int L, const double* Minv, double lambda, RefineConst* rc, uint16_t* tab,
                        cudaStream_t st);
 // initial (or refreshed) field and Green matrices of the chains of one grid
-// (has_U: lambda != 0; mirror: G_dn = 1 - G_up^T instead of its own inversion)
+// (has_U: lambda != 0; mirror: G_dn = 1 - G_up^T instead of its own inversion;
+// n_sm: SMs of the device)
 int launch_init_chains(const SweepArgs& a, const GridConst* d_grid_ptr, int item0, int n_chains,
                        int L, bool f64, bool first_time, bool gj_smem, bool has_U,
-                       bool mirror, cudaStream_t st);
+                       bool mirror, int n_sm, cudaStream_t st);
 // measured-sweep bookkeeping of every grid for one hfqmc_sweep call
 int launch_account(GridAccount* acc, int n_grids, long long n_meas, cudaStream_t st);
 // per-grid mean over chains and error bars

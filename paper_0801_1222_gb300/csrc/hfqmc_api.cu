@@ -775,7 +775,8 @@ int hfqmc_set_G0(hfqmc_ctx* c, int grid, const double* G0_tau) {
   a.status = c->d_status;
   a.seed = c->seed;
   r = launch_init_chains(a, c->d_grids + grid, h.item0, h.chains, h.L, f64_path(c), !h.ever_set,
-                         h.gj_smem != 0, h.lambda != 0.0, h.refine && ph && c->opts.ph_symmetry == 0, c->stream);
+                         h.gj_smem != 0, h.lambda != 0.0, h.refine && ph && c->opts.ph_symmetry == 0, c->n_sm,
+                         c->stream);
   if (r) return cuda_fail(c, (cudaError_t)r, "init kernel");
   CK(cudaMemsetAsync(c->d_account + grid, 0, sizeof(GridAccount), c->stream));
   CK(cudaMemcpyAsync(c->h_status, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));

@@ -303,7 +303,8 @@ size_t init_smem(int L, bool gj_smem) {
 }
 
 int launch_init_chains(const SweepArgs& a, const GridConst* d_grid_ptr, int item0, int n_chains,
-                       int L, bool f64, bool first_time, bool gj_smem, bool has_U, bool mirror, cudaStream_t st) {
+                       int L, bool f64, bool first_time, bool gj_smem, bool has_U, bool mirror, int n_sm,
+                       cudaStream_t st) {
   const size_t sm = init_smem(L, gj_smem);
   cudaError_t e;
   if (!gj_smem && init_blocked(L) && has_U) {
@@ -318,16 +319,20 @@ int launch_init_chains(const SweepArgs& a, const GridConst* d_grid_ptr, int item
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    // The most CTAs per matrix (a portable cluster) for which all matrices are
-    // worked on at once; more would queue behind each other.  np = 1 without
-    // the mirror leaves k_init_chains, whose panel loads need not go to L2 (50
-    // chains at L = 240, both spins: 4.3 ms against 4.7).
+    // The most CTAs per matrix (a portable cluster) for which each has an SM to
+    // itself and all matrices are worked on at once.  CTAs that share an SM
+    // share its FP64 pipe and repeat each other's panel reductions (64 chains
+    // at L = 120, one spin: 0.87 ms with three per matrix, 0.65 with two; 100
+    // matrices at L = 240: 4.7 ms with two, 4.3 by k_init_chains, which np = 1
+    // without the mirror therefore leaves it to).  Not only powers of two: 24
+    // grids of 42 to 46 chains, L = 80 .. 320, take 84 ms with one CTA per
+    // matrix and both spins inverted, 59 with powers of two, 47 with this.
     auto go = [&](auto* f) {
       cudaError_t r = raise_smem_limit(f, sm);
       if (r != cudaSuccess) return (int)r;
       int np = 8;
-      for (; np > 1; np /= 2) {
-        if (L < 32 * np) continue;
+      for (; np > 1; --np) {
+        if (L < 32 * np || np * n_chains * spins > n_sm) continue;
         at[0].val.clusterDim.x = np;
         cfg.gridDim = dim3(n_chains * np, spins);
         int n = 0;
