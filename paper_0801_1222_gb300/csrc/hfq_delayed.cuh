@@ -238,10 +238,20 @@ struct TcState {
 };
 
 // The refinement's counters, kept in shared memory between recomputes: H'
-// buffers and update stages used so far, table copies so far
+// buffers and update stages used so far (see rf_uses), table copies so far
 struct RfSync {
   uint32_t cc, c2, ct;
 };
+
+// A count of uses of bufs buffers in turn, as it is kept: use n takes buffer n
+// % bufs, waits (n >= bufs) for use n - bufs and finds its mbarrier at parity
+// n / bufs % 2.  Only n modulo 2 bufs and whether a buffer was used before
+// matter, so a count is kept below 4 bufs; left to run it would wrap after 2^32
+// uses (some 10^7 sweeps of one call at Lambda = 240), and the first uses after
+// that would not wait for a buffer the tensor cores still read.
+__host__ __device__ constexpr uint32_t rf_uses(uint32_t n, uint32_t bufs) {
+  return n < 2 * bufs ? n : 2 * bufs + n % (2 * bufs);
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);

@@ -566,7 +566,7 @@ __device__ __forceinline__ float rf_product(RfPar& P, const unsigned char* sm, i
     tc_fence_before();
     __syncthreads();
   }
-  if (tid == 0) P.sync.cc = cc + (uint32_t)(nmb * nib) * (uint32_t)(NJ / 2);
+  if (tid == 0) P.sync.cc = rf_uses(cc + (uint32_t)(nmb * nib) * (uint32_t)(NJ / 2), kRfBufs);
   return emax;
 }
 
@@ -803,7 +803,7 @@ __device__ __forceinline__ float rf_update(RfPar& P, unsigned char* sm, int eh, 
       }
     __syncthreads();
   }
-  if (tid == 0) P.sync.c2 = c2;
+  if (tid == 0) P.sync.c2 = rf_uses(c2, 2);
   return drift;
 }
 
