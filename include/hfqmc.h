@@ -300,11 +300,15 @@ int hfqmc_put_trace(hfqmc_ctx *ctx, int grid, const uint32_t *bits, int64_t n_wo
  *   G_up, G_dn  L x L doubles each, row-major, written
  *   cuda_stream  cudaStream_t to run on (NULL: the legacy default stream)
  *   status_out   optional host int: the device status bits of this call
+ * G0_tau may lie inside G_up or G_dn and s inside G_dn: they are overwritten,
+ * after they have been read.  Where G_up and G_dn overlap, G_dn is written last.
+ * A call with overlapping buffers runs as one CTA (several times as long).
  * 1 <= L <= HFQMC_NOALLOC_MAX_L; larger L returns HFQMC_EINVAL before any
  * device work.  The call returns after its work on cuda_stream is done:
  * HFQMC_OK, HFQMC_ENUMERIC (zero pivot or non-finite G), HFQMC_ECUDA.
  *
- * Memory: the [A | M] workspace lives in shared memory while it fits (L <= 159),
+ * Memory: the [A | M] workspace lives in shared memory while it fits (L <= 159)
+ * and no two buffers overlap,
  * else with the bath matrix in one file-scope device array of 3 *
  * HFQMC_NOALLOC_MAX_L^2 doubles (1.5 MiB) that every GPU which loads the
  * library holds until the process exits (the status words are always there).

@@ -10,6 +10,7 @@
 // their own device buffers for the inputs and outputs; the bath matrix and
 // the Gauss-Jordan workspace live in shared memory or in the file-scope array below.
 #include <cmath>
+#include <cstdint>
 
 #include <cuda_runtime.h>
 
@@ -93,7 +94,8 @@ __global__ void __launch_bounds__(kNoAllocNT) k_green_noalloc_shares(GridConst g
   if (tid == 0) *st = bad ? kStatusNonFinite : 0;
 }
 
-// The workspace in the scratch array (M, then [A | M]), one CTA, both spins.
+// The workspace in the scratch array (M, then [A | M]), one CTA, both spins in
+// turn: G0_tau is read before G_up is written, s before G_dn, G_dn last.
 __global__ void __launch_bounds__(kNoAllocNT) k_green_noalloc(GridConst gc, const double* G0_tau,
                                                               const int8_t* s, double* Gup,
                                                               double* Gdn, double* scratch) {
@@ -144,8 +146,18 @@ extern "C" int hfqmc_green_noalloc(const double* G0_tau, const int8_t* s, int L,
   gc.dV[1] = std::exp(-gc.lambda) - 1.0;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   double* status_addr = scratch + 3 * (size_t)kNoAllocMaxL * kNoAllocMaxL;
+  // The shares read G0_tau and s while others already write, in no order: where
+  // a buffer overlaps another, one CTA takes the call, in the order stated there
+  const size_t gbytes = sizeof(double) * (size_t)L * L;
+  const auto overlap = [](const void* a, size_t na, const void* b, size_t nb) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + nb && y < x + na;
+  };
+  bool apart = !overlap(G_up, gbytes, G_dn, gbytes);
+  for (const double* G : {G_up, G_dn})
+    apart = apart && !overlap(G, gbytes, G0_tau, sizeof(double) * L) && !overlap(G, gbytes, s, L);
   int n_words = 1;
-  if (noalloc_shared(L)) {
+  if (apart && noalloc_shared(L)) {
     if (raise_smem_limit(k_green_noalloc_shares, noalloc_smem(L)) != cudaSuccess) return HFQMC_ECUDA;
     n_words = 2 * kNoAllocShares;
     k_green_noalloc_shares<<<dim3(kNoAllocShares, 2), kNoAllocNT, noalloc_smem(L), st>>>(

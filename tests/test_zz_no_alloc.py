@@ -52,3 +52,36 @@ def test_noalloc_rejects_sizes_beyond_the_maximum():
         hfqmc.hfqmc_green_noalloc(buf.data_ptr(), buf.data_ptr(), L, 0.1, 4.0, buf.data_ptr(),
                                   buf.data_ptr(), 0)
     assert ei.value.name == "EINVAL"
+
+
+# buffers that overlap: G0_tau inside either output, s inside G_dn, both
+# outputs the same; by 16 CTAs (L <= 159) each would read what another writes
+@pytest.mark.parametrize("L", [16, 100, 159, 160])
+@pytest.mark.parametrize("where", ["G0 in G_up", "G0 in G_dn", "G0 at the end of G_up", "s in G_dn", "G_up is G_dn"])
+def test_noalloc_overlapping_buffers(L, where):
+    import torch
+
+    from paper_0801_1222_gb300 import build, hfqmc, inputs
+    build.build()
+    dtau, U = 0.2, 5.0
+    g0 = _dev(inputs.bethe_G0_tau(dtau * L, L))
+    s = _dev(np.where(np.random.default_rng(L).random(L) < 0.5, 1, -1).astype(np.int8))
+    ref = [torch.empty((L, L), dtype=torch.float64, device="cuda") for _ in range(2)]
+    out = [torch.empty((L, L), dtype=torch.float64, device="cuda") for _ in range(2)]
+    hfqmc.hfqmc_green_noalloc(g0.data_ptr(), s.data_ptr(), L, dtau, U, ref[0].data_ptr(), ref[1].data_ptr(), 0)
+    g0_p, s_p = g0.data_ptr(), s.data_ptr()
+    if where == "G_up is G_dn":
+        out[0] = out[1]
+    elif where == "s in G_dn":
+        view = out[1].view(-1).view(torch.int8)[8:8 + L]
+        view.copy_(s)
+        s_p = view.data_ptr()
+    else:
+        flat = out[1 if "dn" in where else 0].view(-1)
+        view = flat[L * L - L:] if "end" in where else flat[:L]
+        view.copy_(g0)
+        g0_p = view.data_ptr()
+    torch.cuda.synchronize()
+    assert hfqmc.hfqmc_green_noalloc(g0_p, s_p, L, dtau, U, out[0].data_ptr(), out[1].data_ptr(), 0) == 0
+    for sp in (1,) if where == "G_up is G_dn" else (0, 1):
+        assert torch.max(torch.abs(out[sp] - ref[sp])) <= 1e-10 * torch.max(torch.abs(ref[sp]))
