@@ -343,10 +343,17 @@ __device__ __forceinline__ float rf_scale(const RfPar& P, float* red) {
 // H' = TMEM lanes, kRfN rows i of A); returns this thread's max |E|, sets
 // W.bad on a wait that gave up (then every thread returns early, together).
 // sm: A's table, then the row factors fs (zero beyond L).
+// kAhead4: the read-out's entries of G are loaded four rows ahead instead of all
+// 16 before it.  For the two-spin sweep, whose accept loop the compiler spills
+// registers of for what is live here: with it, and the other cuts marked in
+// k_delayed.cu, 40 two-spin chains at Lambda = 240 without a recompute take 7.9
+// ms for 26 sweeps instead of 11.8.  The one-spin kernel is faster without
+// (15.7 against 16.8 ms for 160 chains at Lambda = 240, 20 sweeps).
 //
 // The cutting warps run through the contraction blocks of all tiles as one
 // stream (a quarter's blocks dealt round its warps), up to kRfAhead K steps
 // into the next tile before they turn to a tile's read-out.
+template <bool kAhead4>
 __device__ __forceinline__ float rf_product(RfPar& P, const unsigned char* sm, int sh, RfWait& W) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = (int)rf_uniform((uint32_t)tid >> 5);  // see elect_one
@@ -474,16 +481,17 @@ __device__ __forceinline__ float rf_product(RfPar& P, const unsigned char* sm, i
     const int ie = tile % nib * kRfN + 16 * g4, n = tile / nib * 128 + 32 * q4 + lane;
     const unsigned neg = __ballot_sync(
         0xffffffffu, lane < 16 && ie + lane < L && P.sig * P.s[ie + lane < L ? ie + lane : 0] < 0);
-    float gd[16];
-    {
-      const float* p = P.G + (size_t)min(ie, L - 1) * P.ld + min(n, L - 1);
+    float gd[kAhead4 ? 4 : 16];
+    auto load_gd = [&](int c0) {  // rows ie + c0 and on
+      const float* p = P.G + (size_t)min(ie + c0, L - 1) * P.ld + min(n, L - 1);
       const int ld = P.ld;
 #pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        if (neg >> c & 1u) gd[c] = *p;  // warp-uniform
+      for (int c = 0; c < (kAhead4 ? 4 : 16); ++c) {
+        if (neg >> (c0 + c) & 1u) gd[c] = *p;  // warp-uniform
         p += ld;
       }
-    }
+    };
+    load_gd(0);
     if (!__syncthreads_and(W.bad ? 0 : 1)) {
       W.bad = true;
       return emax;
@@ -508,6 +516,12 @@ __device__ __forceinline__ float rf_product(RfPar& P, const unsigned char* sm, i
       const int i0 = ie + 4 * h4;
       if (i0 < L) {  // warp-uniform
         const uint32_t ta = lane_base + (uint32_t)(16 * g4 + 4 * h4);
+        float g4r[4];
+        if constexpr (kAhead4) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) g4r[c] = gd[c];
+          if (h4 < 3) load_gd(4 * h4 + 4);
+        }
         uint32_t u[kRfLevels][4];
 #pragma unroll
         for (int lv = 0; lv < kRfLevels; ++lv) tmem_ld4_nowait(ta + (uint32_t)(lv * kRfN), u[lv]);
@@ -521,7 +535,7 @@ __device__ __forceinline__ float rf_product(RfPar& P, const unsigned char* sm, i
 #pragma unroll
           for (int lv = 0; lv < kRfLevels; ++lv) S[lv] = __uint_as_float(u[lv][c]);
           if (neg >> (4 * h4 + c) & 1u) {  // warp-uniform: the other value of A_ii
-            float y = gd[4 * h4 + c] * fs[i0 + c];
+            float y = (kAhead4 ? g4r[c] : gd[kAhead4 ? 0 : 4 * h4 + c]) * fs[i0 + c];
 #pragma unroll
             for (int q = 0; q < kRfSlicesH; ++q) {
               const float d = (y + 12582912.f) - 12582912.f;
@@ -817,6 +831,7 @@ __device__ __forceinline__ float rf_update(RfPar& P, unsigned char* sm, int eh, 
 // Returns the largest change of an entry (>= 0), or -1 if the caller must
 // recompute from scratch (|E| too large, scale out of range, or a wait gave
 // up, which also sets kStatusTimeout).  All threads call it.
+template <bool kAhead4>
 __device__ __forceinline__ float refine_spin(const GridConst& gc, const RefineConst* rc, const int8_t* s, int sig,
                                              float* G, int ld, float* ws, unsigned char* sm0, TcState* tc,
                                              RfSync* sync, float* red, int* status) {
@@ -859,7 +874,7 @@ __device__ __forceinline__ float refine_spin(const GridConst& gc, const RefineCo
       break;
     }
     if (!ok) break;
-    emax = rf_product(P, sm, sh, W);
+    emax = rf_product<kAhead4>(P, sm, sh, W);
     if (W.bad) break;
     emax = rf_block_max(emax, red);
     ok = emax <= P.rc->emax_step;  // else too far for Newton steps (default 2^-8)

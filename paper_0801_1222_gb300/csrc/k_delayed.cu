@@ -367,33 +367,37 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
               }
             }
           };
-          if (resident)
-            base_entries(reinterpret_cast<const float*>(smem + lay.off_G) + (sp && !kMirror ? L * ld : 0), ld);
+          // one spin: G in shared memory and in HBM told apart in the code; two:
+          // one copy through the general pointer, their kernel spills more with two
+          if constexpr (!kMirror)
+            base_entries(Gs, ld);
+          else if (resident)
+            base_entries(reinterpret_cast<const float*>(smem + lay.off_G), ld);
           else
-            base_entries(Ggl + (sp && !kMirror ? L * L : 0), L);
+            base_entries(Ggl, L);
 #pragma unroll
           for (int qq = 0; qq < kRowsPerThread; ++qq) {
             if (qq * kRowStride >= L) break;  // uniform: rows beyond the grid
             const int i0 = row0 + qq * kRowStride, i = min(i0, L - 1);
             const int oi = i * KP, ol = l * KP;  // 32-bit shared-memory offsets
-            // the panels are zero past column j: whole groups of eight columns
-            const int j8 = (j + 7) >> 3;
             float c4[4] = {0.f, 0.f, 0.f, 0.f};
-            auto dot = [&](const float4* x, const float4* y, float* acc) {
-#pragma unroll 1
-              for (int m = 0; m < j8; ++m) {
-                const float4 a1 = x[2 * m], b1 = y[2 * m], a2 = x[2 * m + 1], b2 = y[2 * m + 1];
-                acc[0] = __fmaf_rn(a1.x, b1.x, acc[0]);
-                acc[1] = __fmaf_rn(a1.y, b1.y, acc[1]);
-                acc[2] = __fmaf_rn(a1.z, b1.z, acc[2]);
-                acc[3] = __fmaf_rn(a1.w, b1.w, acc[3]);
-                acc[0] = __fmaf_rn(a2.x, b2.x, acc[0]);
-                acc[1] = __fmaf_rn(a2.y, b2.y, acc[1]);
-                acc[2] = __fmaf_rn(a2.z, b2.z, acc[2]);
-                acc[3] = __fmaf_rn(a2.w, b2.w, acc[3]);
-              }
-            };
             if constexpr (kMirror) {
+              // the panels are zero past column j: whole groups of eight columns
+              const int j8 = (j + 7) >> 3;
+              auto dot = [&](const float4* x, const float4* y, float* acc) {
+#pragma unroll 1
+                for (int m = 0; m < j8; ++m) {
+                  const float4 a1 = x[2 * m], b1 = y[2 * m], a2 = x[2 * m + 1], b2 = y[2 * m + 1];
+                  acc[0] = __fmaf_rn(a1.x, b1.x, acc[0]);
+                  acc[1] = __fmaf_rn(a1.y, b1.y, acc[1]);
+                  acc[2] = __fmaf_rn(a1.z, b1.z, acc[2]);
+                  acc[3] = __fmaf_rn(a1.w, b1.w, acc[3]);
+                  acc[0] = __fmaf_rn(a2.x, b2.x, acc[0]);
+                  acc[1] = __fmaf_rn(a2.y, b2.y, acc[1]);
+                  acc[2] = __fmaf_rn(a2.z, b2.z, acc[2]);
+                  acc[3] = __fmaf_rn(a2.w, b2.w, acc[3]);
+                }
+              };
               // spin up only: the even thread of a pair appends u_i (column l),
               // the odd one w_i (row l); one shuffle gives both the pair's values.
               // Even lane: U row i . W row l; odd lane: W row i . U row l.  The
@@ -412,9 +416,24 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
               }
             } else {
               // append column j of the panels for the owned rows of this thread's spin
+              // (both dot products in one loop, four columns a pass: eight
+              // accumulators hide the latency that two loops in turn wait for)
               float r4[4] = {0.f, 0.f, 0.f, 0.f};
-              dot(reinterpret_cast<const float4*>(Us + oi), reinterpret_cast<const float4*>(Ws + ol), c4);
-              dot(reinterpret_cast<const float4*>(Us + ol), reinterpret_cast<const float4*>(Ws + oi), r4);
+              const float4 *Ui = reinterpret_cast<const float4*>(Us + oi), *Wl = reinterpret_cast<const float4*>(Ws + ol);
+              const float4 *Ul = reinterpret_cast<const float4*>(Us + ol), *Wi = reinterpret_cast<const float4*>(Ws + oi);
+              const int j4 = (j + 3) >> 2;
+#pragma unroll 1
+              for (int m = 0; m < j4; ++m) {
+                const float4 a1 = Ui[m], b1 = Wl[m], a2 = Ul[m], b2 = Wi[m];
+                c4[0] = __fmaf_rn(a1.x, b1.x, c4[0]);
+                c4[1] = __fmaf_rn(a1.y, b1.y, c4[1]);
+                c4[2] = __fmaf_rn(a1.z, b1.z, c4[2]);
+                c4[3] = __fmaf_rn(a1.w, b1.w, c4[3]);
+                r4[0] = __fmaf_rn(a2.x, b2.x, r4[0]);
+                r4[1] = __fmaf_rn(a2.y, b2.y, r4[1]);
+                r4[2] = __fmaf_rn(a2.z, b2.z, r4[2]);
+                r4[3] = __fmaf_rn(a2.w, b2.w, r4[3]);
+              }
               const float uu = gc_q[qq] + ((c4[0] + c4[1]) + (c4[2] + c4[3])) - ((i == l) ? 1.f : 0.f);
               const float ww = (gr_q[qq] + ((r4[0] + r4[1]) + (r4[2] + r4[3]))) * f;
               if (i0 < L) {
@@ -443,12 +462,12 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
         if (j == K) flush();
         if (--left == 0) break;
       }
-      if (left == 0) {
-        flush();
-        break;
-      }
+      // before a recompute, a measurement or the end: one flush in the code for
+      // the three (with one each the kernels spill about twice as much; 40
+      // half-filled chains at Lambda = 500, 15 sweeps, take 18.0 ms instead of 14.3)
+      if (left == 0 || sw >= n_warm || sw + 1 == n_sweeps) flush();
+      if (left == 0) break;
       if (sw >= n_warm) {
-        flush();
         const long long m = sw - n_warm;
         const int b = (int)((kBins * m) / a.n_meas);
         // partial sums in the (idle) staging area, totals in the panels' space
@@ -496,7 +515,6 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
       const int nb = __reduce_add_sync(0xffffffffu, n_bad);
       if (lane == 0 && nb) atomicAdd(&s_bad, nb);
     }
-    flush();
     if (tid == 0) {
       s_pos.n_acc += stretch - left;
       s_pos.sw = sw;
@@ -543,7 +561,7 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
       float dmax = 0.f;
 #pragma unroll 1
       for (int r = 0; r < n_ref && dmax >= 0.f; ++r) {
-        const float dr = refine_spin(gc, gc.rc, ss, r ? -1 : 1, r ? Rd : Ru, rld, rws, smem + lay.off_rf, &tc, &s_rf,
+        const float dr = refine_spin<!kMirror>(gc, gc.rc, ss, r ? -1 : 1, r ? Rd : Ru, rld, rws, smem + lay.off_rf, &tc, &s_rf,
                                      rred, a.status);
         dmax = dr < 0.f ? -1.f : fmaxf(dmax, dr);
       }
