@@ -193,8 +193,11 @@ __device__ __forceinline__ void reset_chain(const ItemPtrs& ip, int L, int first
 // Initial (or, after a new bath, rebuilt) Green matrices of every chain of a
 // grid: block (chain, spin), so the two spins of a chain are inverted by two
 // CTAs at once.  The spin-up block also resets the chain's accumulators.
+// At most 85 registers, for three CTAs per SM (101 without the bound): 200
+// chains at L = 170, both spins, are 400 CTAs on 152 SMs and take 4.3 ms, with
+// two per SM in two waves 6.0.
 template <typename T>
-__global__ void __launch_bounds__(256) k_init_chains(SweepArgs a, const GridConst* gptr, int item0,
+__global__ void __launch_bounds__(256, 3) k_init_chains(SweepArgs a, const GridConst* gptr, int item0,
                                                      int first_time) {
   constexpr int NT = 256;
   extern __shared__ __align__(16) unsigned char dsm[];
