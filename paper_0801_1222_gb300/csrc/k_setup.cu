@@ -4,6 +4,8 @@
 //  * per-call measured-sweep bookkeeping;
 //  * per-grid mean over chains and error bars (the paper averages each grid's
 //    Green function over 10 to 20 impurity solutions, "Multigrid HF-QMC method").
+#include <algorithm>
+
 #include <cuda_fp16.h>
 
 #include "hfq_device.cuh"
@@ -330,10 +332,18 @@ int launch_init_chains(const SweepArgs& a, const GridConst* d_grid_ptr, int item
     // without the mirror therefore leaves it to).  Not only powers of two: 24
     // grids of 42 to 46 chains, L = 80 .. 320, take 84 ms with one CTA per
     // matrix and both spins inverted, 59 with powers of two, 47 with this.
+    // A cluster lies within one GPC, whose SMs need not divide by np: how many
+    // fit is asked for CTAs that take more than half an SM's shared memory, so
+    // that no two count as fitting on one.  With the number of SMs alone as the
+    // limit, the left-over clusters doubled up: 50 matrices at L = 100 took 0.69
+    // ms with three CTAs each, 0.54 with two (0.62 by k_init_chains); 30 at
+    // L = 256 3.1 with five, 1.9 with four.
+    const size_t alone = std::max(sm, (size_t)116 * 1024);
     auto go = [&](auto* f) {
-      cudaError_t r = raise_smem_limit(f, sm);
+      cudaError_t r = raise_smem_limit(f, alone);
       if (r != cudaSuccess) return (int)r;
       int np = 8;
+      cfg.dynamicSmemBytes = alone;
       for (; np > 1; --np) {
         if (L < 32 * np || np * n_chains * spins > n_sm) continue;
         at[0].val.clusterDim.x = np;
@@ -342,6 +352,7 @@ int launch_init_chains(const SweepArgs& a, const GridConst* d_grid_ptr, int item
         if (cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess) (void)cudaGetLastError();
         if (n >= n_chains * spins) break;
       }
+      cfg.dynamicSmemBytes = sm;
       if (np == 1 && !mirror) return -1;
       at[0].val.clusterDim.x = np;
       cfg.gridDim = dim3(n_chains * np, spins);

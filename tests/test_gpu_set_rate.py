@@ -35,3 +35,11 @@ def _set_ms(L, chains, precision, symmetric):
 def test_three_initial_matrices_per_sm(L):
     two, three = (_set_ms(L, chains, "f64_rank1", False) for chains in (152, 200))
     assert three <= 1.65 * two, (two, three)
+
+
+# a chain more has to take a smaller cluster (3 x 51 and 5 x 31 CTAs are more
+# than 152); one less must not take longer because its clusters share SMs
+@pytest.mark.parametrize("L,chains", [(100, 50), (200, 50), (256, 30)])
+def test_clusters_do_not_share_sms(L, chains):
+    here, more = (_set_ms(L, n, "f32_delayed", True) for n in (chains, chains + 1))
+    assert here <= 1.12 * more, (here, more)
