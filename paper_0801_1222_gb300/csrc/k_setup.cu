@@ -195,11 +195,12 @@ __device__ __forceinline__ void reset_chain(const ItemPtrs& ip, int L, int first
 // Initial (or, after a new bath, rebuilt) Green matrices of every chain of a
 // grid: block (chain, spin), so the two spins of a chain are inverted by two
 // CTAs at once.  The spin-up block also resets the chain's accumulators.
-// At most 85 registers, for three CTAs per SM (101 without the bound): 200
-// chains at L = 170, both spins, are 400 CTAs on 152 SMs and take 4.3 ms, with
-// two per SM in two waves 6.0.
-template <typename T>
-__global__ void __launch_bounds__(256, 3) k_init_chains(SweepArgs a, const GridConst* gptr, int item0,
+// kCtas: CTAs per SM that the registers are bounded for. Three (80 registers)
+// where as many are needed and fit: 200 chains at L = 170, both spins, are 400
+// CTAs on 152 SMs and take 4.3 ms, with two per SM in two waves 6.0. Otherwise
+// unbounded, which is 1 % faster per CTA.
+template <typename T, int kCtas>
+__global__ void __launch_bounds__(256, kCtas) k_init_chains(SweepArgs a, const GridConst* gptr, int item0,
                                                      int first_time) {
   constexpr int NT = 256;
   extern __shared__ __align__(16) unsigned char dsm[];
@@ -311,7 +312,6 @@ int launch_init_chains(const SweepArgs& a, const GridConst* d_grid_ptr, int item
                        int L, bool f64, bool first_time, bool gj_smem, bool has_U, bool mirror, int n_sm,
                        cudaStream_t st) {
   const size_t sm = init_smem(L, gj_smem);
-  cudaError_t e;
   if (!gj_smem && init_blocked(L) && has_U) {
     const int spins = mirror ? 1 : 2;
     cudaLaunchConfig_t cfg = {};
@@ -361,16 +361,16 @@ int launch_init_chains(const SweepArgs& a, const GridConst* d_grid_ptr, int item
     const int r = f64 ? go(k_init_chains_cluster<double>) : go(k_init_chains_cluster<float>);
     if (r >= 0) return r;
   }
-  if (f64) {
-    e = cudaFuncSetAttribute(k_init_chains<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  const auto go1 = [&](auto* f) {
+    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return (int)e;
-    k_init_chains<double><<<dim3(n_chains, 2), 256, sm, st>>>(a, d_grid_ptr, item0, first_time ? 1 : 0);
-  } else {
-    e = cudaFuncSetAttribute(k_init_chains<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return (int)e;
-    k_init_chains<float><<<dim3(n_chains, 2), 256, sm, st>>>(a, d_grid_ptr, item0, first_time ? 1 : 0);
-  }
-  return (int)cudaGetLastError();
+    f<<<dim3(n_chains, 2), 256, sm, st>>>(a, d_grid_ptr, item0, first_time ? 1 : 0);
+    return (int)cudaGetLastError();
+  };
+  // three per SM: 228 KB of shared memory, 1 KB of it reserved per CTA
+  const bool three = n_chains > n_sm && 3 * (sm + 1024) <= 228 * 1024;
+  if (f64) return three ? go1(k_init_chains<double, 3>) : go1(k_init_chains<double, 1>);
+  return three ? go1(k_init_chains<float, 3>) : go1(k_init_chains<float, 1>);
 }
 
 // Measured sweep m (0-based within one call of n_meas) goes to bin floor(32 m / n_meas);
