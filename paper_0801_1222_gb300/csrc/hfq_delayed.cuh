@@ -169,16 +169,6 @@ __device__ __forceinline__ bool del_decide(float d0, float d1, float gu, float g
   return rule == 0 ? (u < R) : (__fmul_rn(u, __fadd_rn(1.f, R)) < R);
 }
 
-__device__ __forceinline__ void del_factors(float d0, float d1, float gu, float gd, int sl, float* fu,
-                                            float* fd) {
-  const float du = sl > 0 ? d0 : d1;
-  const float dd = sl > 0 ? d1 : d0;
-  const float Ru = __fadd_rn(1.f, __fmul_rn(__fsub_rn(1.f, gu), du));
-  const float Rd = __fadd_rn(1.f, __fmul_rn(__fsub_rn(1.f, gd), dd));
-  *fu = du / Ru;
-  *fd = dd / Rd;
-}
-
 // ---------------------------------------------------------------------------
 // FP32 FMA flush: G^sigma[i][c] += sum_{m<j} U^sigma[i][m] W^sigma[c][m]
 // ---------------------------------------------------------------------------
@@ -422,7 +412,6 @@ __device__ __forceinline__ void tma_reduce_add_4d(const void* tmap, uint32_t src
       : "memory");
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 

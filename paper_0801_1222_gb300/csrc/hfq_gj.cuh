@@ -11,8 +11,8 @@
 //  * recompute_green_inv: G = B^{-1} with B = M^{-1}(1 + D) - D inverted in
 //    place, L^3 DFMA per spin on an L x L workspace.  Used by every sweep
 //    kernel and the initialisation.  Two forms of the inversion:
-//    gj_invert_inplace (row interchanges; three barriers per pivot column:
-//    search, swap + scale, elimination) on a workspace in shared memory
+//    gj_invert_inplace (row interchanges; four barriers per pivot column: two
+//    in the search, swap + scale, elimination) on a workspace in shared memory
 //    (rank-1 paths and initialisation, Lambda <= 168) or in HBM when nothing
 //    else fits; gj_invert_blocked (implicit pivoting, kGjPanel columns per
 //    panel in shared memory, two barriers per pivot column) on the chain's

@@ -832,15 +832,15 @@ __device__ __forceinline__ float rf_update(RfPar& P, unsigned char* sm, int eh, 
 // recompute from scratch (|E| too large, scale out of range, or a wait gave
 // up, which also sets kStatusTimeout).  All threads call it.
 template <bool kAhead4>
-__device__ __forceinline__ float refine_spin(const GridConst& gc, const RefineConst* rc, const int8_t* s, int sig,
-                                             float* G, int ld, float* ws, unsigned char* sm0, TcState* tc,
-                                             RfSync* sync, float* red, int* status) {
+__device__ __forceinline__ float refine_spin(int L, const RefineConst* rc, const int8_t* s, int sig, float* G, int ld,
+                                             float* ws, unsigned char* sm0, TcState* tc, RfSync* sync, float* red,
+                                             int* status) {
   RfPar& P = *reinterpret_cast<RfPar*>(sm0);
   unsigned char* sm = sm0 + kRfParBytes;
   // what the region held before was read and written through the generic proxy
   fence_async_smem();
   __syncthreads();
-  if (threadIdx.x == 0) P = RfPar{G, ws, rc, s, status, gc.L, ld, sig, tc->tmem, tc->cbar, *sync};
+  if (threadIdx.x == 0) P = RfPar{G, ws, rc, s, status, L, ld, sig, tc->tmem, tc->cbar, *sync};
   __syncthreads();
   RfWait W;
   float drift = 0.f, emax = 0.f;

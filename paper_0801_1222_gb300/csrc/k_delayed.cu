@@ -25,7 +25,7 @@
 // the minimum of the slots and each thread divides for its flip factor while
 // G's column and row are on their way.  (With one atomicMin for all warps, the
 // division before the barrier and a branch around every load, 256 chains at
-// Lambda = 100 took 86 ms for 550 sweeps; they take 75.)
+// Lambda = 100 took 86 ms for 550 sweeps; they take 69.)
 #include "hfq_delayed.cuh"
 #include "hfq_device.cuh"
 #include "hfq_gj.cuh"
@@ -561,8 +561,8 @@ __global__ void __launch_bounds__(kDelNT, 1) k_sweep_delayed(SweepArgs a) {
       float dmax = 0.f;
 #pragma unroll 1
       for (int r = 0; r < n_ref && dmax >= 0.f; ++r) {
-        const float dr = refine_spin<!kMirror>(gc, gc.rc, ss, r ? -1 : 1, r ? Rd : Ru, rld, rws, smem + lay.off_rf, &tc, &s_rf,
-                                     rred, a.status);
+        const float dr = refine_spin<!kMirror>(L, gc.rc, ss, r ? -1 : 1, r ? Rd : Ru, rld, rws, smem + lay.off_rf, &tc,
+                                               &s_rf, rred, a.status);
         dmax = dr < 0.f ? -1.f : fmaxf(dmax, dr);
       }
       if (!kMirror && gc.ph && dmax >= 0.f)
