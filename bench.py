@@ -46,7 +46,7 @@ LONG_NWRAP_TABLE = [(64, 32, 8192), (128, 32, 8192), (144, 32, 16384), (176, 24,
 # dram read + write of one full-size launch (1000 sweeps of the multigrid
 # workload at N_wrap 64), from a one-pass ncu capture of this kernel (None
 # while the kernel has changed since)
-TRAFFIC_PER_1000_SWEEPS = 550386944 + 39742442496
+TRAFFIC_PER_1000_SWEEPS = 238025216 + 27051183616
 
 
 def parse():

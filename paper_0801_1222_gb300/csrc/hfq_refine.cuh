@@ -62,10 +62,10 @@
 //
 // SM cycles per refinement of one spin at Lambda = 240 (phase timers in a copy
 // of the kernel), with A's slices streamed from L2 and H' cut into shared
-// memory, and as it is here: residual product 180k -> 117k (its MMAs alone
+// memory, and as it is here: residual product 180k -> 122k (its MMAs alone
 // take 69k; what is above is the hand-over between the cutting and the issuing
-// warps), its read-outs 50k -> 39k, update product 46k -> 34k, its read-out
-// 31k -> 26k, scale pass 16k -> 13k; at Lambda = 500 in all 2.83M -> 1.85M.
+// warps), its read-outs 50k -> 35k, update product 46k -> 32k, its read-out
+// 31k -> 21k, scale pass 16k -> 10k; at Lambda = 500 in all 2.83M -> 1.81M.
 // Measured and not kept for Lambda > 256: H' and E^T written once as FP16
 // parts and staged by bulk copies (the chains' working set is beyond L2 there:
 // 673k cycles for the update product instead of 495k).
