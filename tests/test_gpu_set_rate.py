@@ -19,7 +19,7 @@ def _set_ms(L, chains, precision, symmetric):
         g0 = g0 * np.exp(-0.3 * np.arange(L) / L)
     ctx = lib().HFQMC(beta, 4.0, [0.2], [chains], seed=11, precision=precision)
     t = []
-    for _ in range(8):
+    for _ in range(20):
         t0 = time.perf_counter()
         ctx.set_G0(0, g0)
         t.append((time.perf_counter() - t0) * 1e3)
